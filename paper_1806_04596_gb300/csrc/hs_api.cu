@@ -28,6 +28,8 @@ struct hs_plan {
 // state never shares partial-sum buffers between its two concurrent branches.
 struct hs_pd_state {
     Plan* p = nullptr;
+    std::shared_ptr<Plan> plane;   // whole-plane layout of the data term (FP32 with the nuclear prior)
+    Plan* dp = nullptr;            // layout of the data term: plane or p
     hs_pd_params prm{};
     void* X = nullptr;      // L x N reals: primal estimate
     void* Xt = nullptr;     // L x N: extrapolated 2 X - X_prev
@@ -67,6 +69,13 @@ struct hs_pd_state {
 };
 
 static cudaStream_t S(void* s) { return reinterpret_cast<cudaStream_t>(s); }
+
+// Caller-order value in the plan's order (conjugated where the sample was mirrored).
+template <typename CT> __device__ __forceinline__ CT gather_one(const CT* __restrict__ in, int q) {
+    CT v = in[q & (int)~PERM_MIRROR];
+    if (q < 0) v.y = -v.y;
+    return v;
+}
 
 #define CHECK_PLAN(pl)                                                         \
     do {                                                                       \
@@ -554,13 +563,13 @@ __global__ void k_gather_c2(const float2* __restrict__ in, const int* __restrict
                             float2* __restrict__ out, int64_t n) {
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
          i += (int64_t)gridDim.x * blockDim.x)
-        out[i] = in[perm[i]];
+        out[i] = gather_one(in, perm[i]);
 }
 __global__ void k_gather_z2(const double2* __restrict__ in, const int* __restrict__ perm,
                             double2* __restrict__ out, int64_t n) {
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
          i += (int64_t)gridDim.x * blockDim.x)
-        out[i] = in[perm[i]];
+        out[i] = gather_one(in, perm[i]);
 }
 
 hs_status hs_pd_state_create(hs_plan_t plan, const void* Y, const double* eps,
@@ -587,6 +596,12 @@ hs_status hs_pd_state_create(hs_plan_t plan, const void* Y, const double* eps,
     const size_t rs = p->rsize(), cs = p->csize();
     const int64_t M = p->M_total;
     hs_status e = HS_OK;
+    st->dp = p;
+    if (prm->use_nuclear && p->prec == HS_F32 && M > 0) {
+        HS_TRY(plane_plan(p, &st->plane, s));
+        st->dp = st->plane.get();
+    }
+    Plan* dp = st->dp;
 #define ALLOC(ptr, bytes)                                   \
     do {                                                    \
         e = st_alloc(st.get(), (void**)&(ptr), (bytes));    \
@@ -615,7 +630,7 @@ hs_status hs_pd_state_create(hs_plan_t plan, const void* Y, const double* eps,
     ALLOC(st->beta, sizeof(double));
     st->nprim = 1024;
     ALLOC(st->ppart, 2 * st->nprim * sizeof(double));
-    st->nbx = degrid_items_max(p);   // slots block * nbx + k; slots without a work item stay 0
+    st->nbx = degrid_items_max(dp);   // slots block * nbx + k; slots without a work item stay 0
     ALLOC(st->dpart, (size_t)nb * st->nbx * sizeof(double));
     ALLOC(st->rpart, (size_t)nb * st->nbx * sizeof(double));
     ALLOC(st->warm, (size_t)MAX_L_NUC * MAX_L_NUC * sizeof(float));
@@ -657,8 +672,8 @@ hs_status hs_pd_state_create(hs_plan_t plan, const void* Y, const double* eps,
     }
     if (M > 0) {
         const unsigned g = (unsigned)std::min<int64_t>((M + 255) / 256, 8192);
-        if (p->prec == HS_F32) k_gather_c2<<<g, 256, 0, s>>>((const float2*)Y, p->perm, (float2*)st->y, M);
-        else k_gather_z2<<<g, 256, 0, s>>>((const double2*)Y, p->perm, (double2*)st->y, M);
+        if (p->prec == HS_F32) k_gather_c2<<<g, 256, 0, s>>>((const float2*)Y, st->dp->perm, (float2*)st->y, M);
+        else k_gather_z2<<<g, 256, 0, s>>>((const double2*)Y, st->dp->perm, (double2*)st->y, M);
         HS_TRY(cu(cudaGetLastError(), "gather"));
     }
     HS_TRY(cu(cudaStreamCreateWithFlags(&st->side, cudaStreamNonBlocking), "stream"));
@@ -682,8 +697,8 @@ hs_status hs_pd_set_data(hs_pd_state_t st, const void* Y, const double* eps, voi
     HS_CHECK_CUDA(cudaMemcpyAsync(st->eps, eps, p->nblk * sizeof(double), cudaMemcpyDeviceToDevice, s));
     if (M > 0) {
         const unsigned g = (unsigned)std::min<int64_t>((M + 255) / 256, 8192);
-        if (p->prec == HS_F32) k_gather_c2<<<g, 256, 0, s>>>((const float2*)Y, p->perm, (float2*)st->y, M);
-        else k_gather_z2<<<g, 256, 0, s>>>((const double2*)Y, p->perm, (double2*)st->y, M);
+        if (p->prec == HS_F32) k_gather_c2<<<g, 256, 0, s>>>((const float2*)Y, st->dp->perm, (float2*)st->y, M);
+        else k_gather_z2<<<g, 256, 0, s>>>((const double2*)Y, st->dp->perm, (double2*)st->y, M);
         HS_CHECK_LAUNCH();
     }
     return HS_OK;
@@ -701,8 +716,8 @@ hs_status hs_pd_set_data_host(hs_pd_state_t st, const void* Y_host, const double
     if (M > 0) {
         HS_CHECK_CUDA(cudaMemcpyAsync(st->ystage, Y_host, (size_t)M * p->csize(), cudaMemcpyHostToDevice, s));
         const unsigned g = (unsigned)std::min<int64_t>((M + 255) / 256, 8192);
-        if (p->prec == HS_F32) k_gather_c2<<<g, 256, 0, s>>>((const float2*)st->ystage, p->perm, (float2*)st->y, M);
-        else k_gather_z2<<<g, 256, 0, s>>>((const double2*)st->ystage, p->perm, (double2*)st->y, M);
+        if (p->prec == HS_F32) k_gather_c2<<<g, 256, 0, s>>>((const float2*)st->ystage, st->dp->perm, (float2*)st->y, M);
+        else k_gather_z2<<<g, 256, 0, s>>>((const double2*)st->ystage, st->dp->perm, (double2*)st->y, M);
         HS_CHECK_LAUNCH();
     }
     return HS_OK;
@@ -756,8 +771,9 @@ static hs_status pd_step_launch(hs_pd_state* st, cudaStream_t s) {
     }
     HS_CHECK_CUDA(cudaEventRecord(st->ev_join2, st->side2));
     // ---- data fidelity (main stream)
+    Plan* dp = st->dp;
     if (p->M_total > 0) {
-        HS_TRY(fft_forward(p, st->Xt, s));                        // step 4
+        HS_TRY(fft_forward(dp, st->Xt, s));                       // step 4
         DegridArgs da{};
         da.mode = DOUT_PD;
         da.v = st->v;
@@ -765,7 +781,7 @@ static hs_status pd_step_launch(hs_pd_state* st, cudaStream_t s) {
         da.d = st->d;
         da.part = st->dpart;
         da.rpart = st->adapt.enable ? st->rpart : nullptr;
-        HS_TRY(degrid(p, da, s));                                  // step 10 (+ residual norms)
+        HS_TRY(degrid(dp, da, s));                                 // step 10 (+ residual norms)
         HS_TRY(ball_scale_from_partials(p, st->dpart, st->nbx, st->eps, st->rho, st->scale, s));
         if (st->adapt.enable) {   // steps 13-19: bounds for the next iteration
             AdaptArgs aa{};
@@ -786,8 +802,8 @@ static hs_status pd_step_launch(hs_pd_state* st, cudaStream_t s) {
         ga.d = st->d;
         ga.scale = st->scale;
         ga.v = st->v;
-        HS_TRY(grid(p, ga, s));                                    // steps 11-12
-        HS_TRY(fft_adjoint(p, st->D, s));                          // Z^T F^H of step 20
+        HS_TRY(grid(dp, ga, s));                                   // steps 11-12
+        HS_TRY(fft_adjoint(dp, st->D, s));                         // Z^T F^H of step 20
     } else {
         HS_CHECK_CUDA(cudaMemsetAsync(st->D, 0, n * p->rsize(), s));
     }

@@ -4,6 +4,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <memory>
+#include <mutex>
 #include <string>
 #include <vector>
 
@@ -67,21 +69,35 @@ constexpr int LR_TOTAL_DOUBLES = LR_DOUBLES + (LRF_G + MAX_L_NUC + 1) / 2;
 // Coordinates of one visibility in an FP64 plan: window start cells and the
 // fractional part of t = u K / (2 pi) (exact in FP64).
 struct Coord64 {
-    double fx, fy;
-    int cx, cy;   // floor(t) mod K per axis
+    double fx, fy;   // in [0, 1] (1 on the mirror image of a sample on a cell)
+    int cx, cy;      // window start column in memory; floor(t) mod Ky
 };
+
+// Half plane: sorted visibilities with u < 0 are kept at the mirrored point (-u, -v), their
+// values conjugated (the image is real, so both describe the same datum): bit
+// 31 of the plan's permutation marks them.
+constexpr unsigned PERM_MIRROR = 0x80000000u;
 
 // Sizes passed by value to kernels.
 struct Geo {
     int nx, ny, L, Kx, Ky;
     int fbx, fby;          // fractional bits of the FP32 fixed-point coordinates
     int tx, ty, ntx, nty;  // gridding tile size and tiles per axis
-    int kxm, kym;          // Kx - 1, Ky - 1 for powers of two, else -1 (wrapn)
+    int kwm, kym;          // Kw - 1, Ky - 1 for powers of two, else -1 (wrapn)
+    // Grid in memory: Kc columns at a pitch of Kw. Half plane: column c holds kx = c - 3,
+    // c < nx + 8 (no window wraps). Whole plane: column c holds kx = c, Kc = Kw = Kx.
+    int Kc, Kw;
 };
 
 // ---------------------------------------------------------------- plan
 struct Plan {
     Geo g{};
+    // Spectrum kept on the half plane kx >= 0 (the image is real), samples with u < 0
+    // mirrored; false: the whole plane (plane_plan).
+    bool half = true;
+    std::vector<float> uv_h;           // uv of FP32 plans the nuclear prior can use (plane_plan)
+    std::weak_ptr<Plan> plane;         // whole-plane layout shared by the states that use it
+    std::mutex plane_mu;
     int levels = 4;
     int J = 8, o = 2;
     hs_prec prec = HS_F32;
@@ -97,7 +113,7 @@ struct Plan {
     int nblk = 0;
     int* blk_id = nullptr;             // block of every sorted visibility (only when nblk != L)
     int64_t* off_d = nullptr;          // L+1
-    int* perm = nullptr;               // sorted index -> caller index
+    int* perm = nullptr;               // sorted index -> caller index (PERM_MIRROR: value conjugated)
     void* coords = nullptr;            // FP32: uint2 fixed point; FP64: Coord64
     void* w_sorted = nullptr;          // Theta in sorted order (real) or null
     void* u_sorted = nullptr;          // U in sorted order (real) or null
@@ -119,6 +135,7 @@ struct Plan {
     int64_t n_sw_ent = 0;
     void* kbc = nullptr;               // 8 * kb_terms reals
     std::vector<double> kbc_h;         // the same on the host
+    std::vector<int> k0x_h, k0y_h;     // window starts in sorted order (while the lists are being built)
     cudaStream_t fft_side = nullptr;   // row passes of a chunked F^H (overlap the next chunk's column pass)
     cudaEvent_t fft_ev_col = nullptr, fft_ev_join = nullptr;
     void* cxs = nullptr;               // nx reals (Z scale along x)
@@ -127,8 +144,8 @@ struct Plan {
     void* twy = nullptr;               // Ky complex
     void* filt = nullptr;              // 8 * 2 * MAXF reals: lowpass, highpass per db_p
     // scratch
-    void* grid = nullptr;              // L * Ky * Kx complex
-    void* tmp = nullptr;               // L * ny * Kx complex
+    void* grid = nullptr;              // L * Ky * Kw complex
+    void* tmp = nullptr;               // L * ny * Kc complex
     void* vis = nullptr;               // M_total complex (sorted order)
     void* dwt_a = nullptr;             // 8 * L * N reals
     void* dwt_b = nullptr;             // 8 * L * N reals
@@ -161,6 +178,19 @@ struct Plan {
     size_t csize() const { return 2 * rsize(); }
 };
 
+// The whole-plane layout of an FP32 plan's coverage (grid, lists, scratch of its own), built on
+// the first call and shared while a state holds it. The iteration with the nuclear prior uses
+// it: its eigensolver, warm-started with at most one Jacobi sweep per iteration, turns last-bit
+// differences of the gradient into 1e-4 of the image over the first ten iterations (256 x 256,
+// L = 60: 5e-6 .. 1.8e-4 between the two Gram forms), so those solves keep the
+// whole-plane summation orders and reproduce their earlier iterates bit for bit.
+hs_status plane_plan(Plan* p, std::shared_ptr<Plan>* out, cudaStream_t s);
+// FFT of the whole plane (hs_fft_plane.cu; FP32).
+hs_status plane_fft_forward(Plan* p, const void* X, cudaStream_t s);
+hs_status plane_fft_cols_inv(Plan* p, const void* grid, void* tmp, int nl, cudaStream_t s);
+hs_status plane_fft_rows_inv(Plan* p, const void* tmp, void* X, int nl, cudaStream_t s);
+hs_status plane_fft_init();
+
 // Device allocation tracked by the plan (freed in destroy).
 hs_status plan_alloc(Plan* p, void** ptr, size_t bytes);
 // Every device allocation of the library goes through these (process-wide
@@ -191,6 +221,7 @@ enum GridIn { GIN_CALLER = 0, GIN_SORTED = 1, GIN_PD = 2 };
 // FFT stages (hs_fft.cu)
 hs_status fft_forward(Plan* p, const void* X, cudaStream_t s);           // X -> p->grid
 hs_status fft_adjoint(Plan* p, void* X, cudaStream_t s);                 // p->grid -> X
+hs_status fft_prepare(Plan* p);                                          // kernel attributes, at creation
 
 // NUFFT interpolation (hs_nufft.cu)
 struct DegridArgs {

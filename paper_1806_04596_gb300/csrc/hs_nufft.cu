@@ -30,7 +30,7 @@ namespace hs {
 
 template <typename R> struct VisCoord;
 template <> struct VisCoord<float> {
-    // fixed point: cell in the high bits, fraction in the low `fb` bits
+    // fixed point: window start column / cell in the high bits, fraction in the low `fb` bits
     static __device__ __forceinline__ void get(const void* c, int64_t i, const Geo& g, int& cxv,
                                                int& cyv, float& fx, float& fy) {
         const uint2 t = ((const uint2*)c)[i];
@@ -50,6 +50,14 @@ template <> struct VisCoord<double> {
         fy = t.fy;
     }
 };
+
+// Caller index of a permutation entry, and a caller's value in the plan's order or
+// back (conjugated where the sample was mirrored).
+__device__ __forceinline__ int perm_index(int p) { return p & (int)~PERM_MIRROR; }
+template <typename CT> __device__ __forceinline__ CT perm_value(int p, CT v) {
+    if (p < 0) v.y = -v.y;
+    return v;
+}
 
 template <typename R> struct NufftK {
     Geo g;
@@ -114,23 +122,23 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 5 : 1)
     const int ntiles = a.g.ntx * a.g.nty;
     const int l = it.tix / ntiles;
     const int t = it.tix - l * ntiles;
-    const int Kx = a.g.Kx, Ky = a.g.Ky;
-    const int kxm = a.g.kxm, kym = a.g.kym;
+    const int Kw = a.g.Kw, Ky = a.g.Ky;
+    const int kwm = a.g.kwm, kym = a.g.kym;
     const int ty0 = (t / a.g.ntx) * a.g.ty, tx0 = (t % a.g.ntx) * a.g.tx;
-    const CT* G = a.grid + (int64_t)l * Ky * Kx;
+    const CT* G = a.grid + (int64_t)l * Ky * Kw;
     if constexpr (sizeof(R) == 4) {
-        // FP32: 16-byte chunks of two cells (tx0 and Kx even: a chunk never straddles the wrap)
+        // FP32: 16-byte chunks of two cells (tx0 and Kw even: a chunk never straddles the wrap)
         constexpr int CPR = DG_REG / 2;   // chunks per staged row
         for (int k = threadIdx.x; k < DG_REG * CPR; k += blockDim.x) {
             const int r = k / CPR, c = 2 * (k - r * CPR);
             const unsigned d = (unsigned)__cvta_generic_to_shared(S + r * DG_LDS + c);
-            const CT* src = G + (int64_t)(wrapn(ty0 + r, Ky, kym)) * Kx + (wrapn(tx0 + c, Kx, kxm));
+            const CT* src = G + (int64_t)(wrapn(ty0 + r, Ky, kym)) * Kw + (wrapn(tx0 + c, Kw, kwm));
             asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(d), "l"(src) : "memory");
         }
     } else {
         for (int k = threadIdx.x; k < DG_REG * DG_REG; k += blockDim.x) {
             const int r = k / DG_REG, c = k - r * DG_REG;
-            cp_async_cx<R>(S + r * DG_LDS + c, G + (int64_t)(wrapn(ty0 + r, Ky, kym)) * Kx + (wrapn(tx0 + c, Kx, kxm)));
+            cp_async_cx<R>(S + r * DG_LDS + c, G + (int64_t)(wrapn(ty0 + r, Ky, kym)) * Kw + (wrapn(tx0 + c, Kw, kwm)));
         }
     }
     asm volatile("cp.async.commit_group;\n" ::: "memory");
@@ -174,7 +182,7 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 5 : 1)
             const R fx = __shfl_sync(0xffffffffu, pfx, src);
             const R fy = __shfl_sync(0xffffffffu, pfy, src);
             // window start relative to the staged region: 0..32 (carry included)
-            const int ox = wrapn(wrapn(cxv - 3, Kx, kxm) - tx0, Kx, kxm);
+            const int ox = wrapn(cxv - tx0, Kw, kwm);
             const int oy = wrapn(wrapn(cyv - 3, Ky, kym) - ty0, Ky, kym);
             off[h] = min(oy, DG_REG - 8) * DG_LDS + min(ox, DG_REG - 8) + j;
             pu[h] = horner<R, NC>(c, (R)2 * fx - (R)1);
@@ -221,7 +229,8 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 5 : 1)
             CT v = mine;
             if (a.w) v = cscale(v, a.w[i]);
             if (MODE == DOUT_CALLER) {
-                a.out[a.perm[i]] = v;
+                const int q = a.perm[i];
+                a.out[perm_index(q)] = perm_value(q, v);
             } else if (MODE == DOUT_SORTED) {
                 a.out[i] = v;
             } else if (MODE == DOUT_SORTED_U) {
@@ -287,8 +296,8 @@ __global__ void __launch_bounds__(GRID_WARPS * 32) k_grid(NufftK<R> a, const Gri
     const int t = it.tix - l * ntiles;
     const int tyi = t / a.g.ntx, txi = t - tyi * a.g.ntx;
     const int ty0 = tyi * TY, tx0 = txi * TX;
-    const int Kx = a.g.Kx, Ky = a.g.Ky;
-    const int kxm = a.g.kxm, kym = a.g.kym;
+    const int Kw = a.g.Kw, Ky = a.g.Ky;
+    const int kwm = a.g.kwm, kym = a.g.kym;
     for (int k = threadIdx.x; k < GRID_WARPS * cells; k += blockDim.x) {
         acc[k] = cx<R>(0, 0);
         if (KAHAN) cmp[k] = cx<R>(0, 0);
@@ -316,11 +325,12 @@ __global__ void __launch_bounds__(GRID_WARPS * 32) k_grid(NufftK<R> a, const Gri
         if (i >= 0) {
             int cxv, cyv;
             VisCoord<R>::get(a.coords, i, a.g, cxv, cyv, fx, fy);
-            const int k0x = wrapn(cxv - 3, Kx, kxm);
+            const int k0x = cxv;
             const int k0y = wrapn(cyv - 3, Ky, kym);
             CT val;
             if (MODE == GIN_CALLER) {
-                val = a.in[a.perm[i]];
+                const int q = a.perm[i];
+                val = perm_value(q, a.in[perm_index(q)]);
             } else if (MODE == GIN_SORTED) {
                 val = a.in[i];
             } else {   // GIN_PD: v = U^{1/2} d max(0, 1 - eps / rho); the home tile stores it
@@ -343,7 +353,7 @@ __global__ void __launch_bounds__(GRID_WARPS * 32) k_grid(NufftK<R> a, const Gri
         for (int k = 0; k < nb; ++k) {
             const int2 b0 = s_k0[w][k];
             if (b0.x < 0) continue;
-            const int gx = (wrapn(b0.x + cc, Kx, kxm)) - tx0;
+            const int gx = (wrapn(b0.x + cc, Kw, kwm)) - tx0;
             if (gx >= 0 && gx < TX) {
                 const CT vv = s_val[w][k];
                 const R pu = s_phi[w][k][cc];
@@ -379,8 +389,8 @@ __global__ void __launch_bounds__(GRID_WARPS * 32) k_grid(NufftK<R> a, const Gri
     CT* Gout;
     int64_t gstride;
     if (it.slot < 0) {
-        Gout = a.grid_out + (int64_t)l * Ky * Kx + (int64_t)ty0 * Kx + tx0;
-        gstride = Kx;
+        Gout = a.grid_out + (int64_t)l * Ky * Kw + (int64_t)ty0 * Kw + tx0;
+        gstride = Kw;
     } else {
         Gout = partial + (int64_t)it.slot * cells;
         gstride = TX;
@@ -439,8 +449,8 @@ __global__ void __launch_bounds__(GRID_PW * 32) k_grid_groups(NufftK<R> a, const
     const int t = it.tix - l * ntiles;
     const int tyi = t / a.g.ntx, txi = t - tyi * a.g.ntx;
     const int ty0 = tyi * TY, tx0 = txi * TX;
-    const int Kx = a.g.Kx, Ky = a.g.Ky;
-    const int kxm = a.g.kxm, kym = a.g.kym;
+    const int Kw = a.g.Kw, Ky = a.g.Ky;
+    const int kwm = a.g.kwm, kym = a.g.kym;
     for (int k = threadIdx.x; k < GRID_PW * TCELLS; k += blockDim.x) priv[k] = cx<R>(0, 0);
     __syncthreads();
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -462,10 +472,11 @@ __global__ void __launch_bounds__(GRID_PW * 32) k_grid_groups(NufftK<R> a, const
             if (i >= 0) {
                 int cxv, cyv;
                 VisCoord<R>::get(a.coords, i, a.g, cxv, cyv, fx, fy);
-                k0x = wrapn(cxv - 3, Kx, kxm);
+                k0x = cxv;
                 k0y = wrapn(cyv - 3, Ky, kym);
                 if (MODE == GIN_CALLER) {
-                    val = a.in[a.perm[i]];
+                    const int q = a.perm[i];
+                    val = perm_value(q, a.in[perm_index(q)]);
                 } else if (MODE == GIN_SORTED) {
                     val = a.in[i];
                 } else {   // GIN_PD: v = U^{1/2} d max(0, 1 - eps / rho); the home tile stores it
@@ -487,7 +498,7 @@ __global__ void __launch_bounds__(GRID_PW * 32) k_grid_groups(NufftK<R> a, const
             if (sx < 0) continue;   // padding; uniform over the 8 lanes of a window
             const R phx = horner<R, NC>(c, (R)2 * sfx - (R)1);   // phi_u of column j
             const R phy = horner<R, NC>(c, (R)2 * sfy - (R)1);   // phi_v of row j
-            const int gx = (wrapn(sx + j, Kx, kxm)) - tx0;
+            const int gx = (wrapn(sx + j, Kw, kwm)) - tx0;
             const bool colok = (unsigned)gx < (unsigned)TX;
             const R pr = phx * vr, pi = phx * vi;
             // the 8 rows of a window are distinct cells: load all, add, store all
@@ -516,8 +527,8 @@ __global__ void __launch_bounds__(GRID_PW * 32) k_grid_groups(NufftK<R> a, const
     CT* Gout;
     int64_t gstride;
     if (it.slot < 0) {
-        Gout = a.grid_out + (int64_t)l * Ky * Kx + (int64_t)ty0 * Kx + tx0;
-        gstride = Kx;
+        Gout = a.grid_out + (int64_t)l * Ky * Kw + (int64_t)ty0 * Kw + tx0;
+        gstride = Kw;
     } else {
         Gout = partial + (int64_t)it.slot * TX * TY;
         gstride = TX;
@@ -593,10 +604,10 @@ __global__ void __launch_bounds__(SW_WARPS * 32, sizeof(R) == 4 ? 5 : 1)
     const int wi = blockIdx.x * SW_WARPS + w;
     if (wi >= n_items) return;
     const SweepItem it = items[wi];
-    const int Kx = a.g.Kx, Ky = a.g.Ky;
-    const int kxm = a.g.kxm, kym = a.g.kym;
+    const int Kw = a.g.Kw, Ky = a.g.Ky;
+    const int kwm = a.g.kwm, kym = a.g.kym;
     const int c0 = it.strip * GRID_TILE, row0 = it.row0, H = it.row1 - it.row0;
-    CT* out = a.grid_out + (int64_t)it.l * Ky * Kx + (int64_t)row0 * Kx + c0 + lane;
+    CT* out = a.grid_out + (int64_t)it.l * Ky * Kw + (int64_t)row0 * Kw + c0 + lane;
     CT B0[4], B1[4], B2[4];
 #pragma unroll
     for (int k = 0; k < 4; ++k) B0[k] = B1[k] = B2[k] = cx<R>(0, 0);
@@ -641,7 +652,7 @@ __global__ void __launch_bounds__(SW_WARPS * 32, sizeof(R) == 4 ? 5 : 1)
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
             const int r = 4 * jb + k;
-            if ((unsigned)r < (unsigned)H) out[(int64_t)r * Kx] = U[k];
+            if ((unsigned)r < (unsigned)H) out[(int64_t)r * Kw] = U[k];
             U[k] = cx<R>(0, 0);
         }
     };
@@ -687,13 +698,13 @@ __global__ void __launch_bounds__(SW_WARPS * 32, sizeof(R) == 4 ? 5 : 1)
             int cxv, cyv;
             R fx, fy;
             VisCoord<R>::get(a.coords, i, a.g, cxv, cyv, fx, fy);
-            const int k0x = wrapn(cxv - 3, Kx, kxm);
+            const int k0x = cxv;
             const int k0y = wrapn(cyv - 3, Ky, kym);
-            const int rx = (wrapn(k0x - c0 + 7, Kx, kxm)) - 7;     // -7 .. 31
+            const int rx = (wrapn(k0x - c0 + 7, Kw, kwm)) - 7;     // -7 .. 31
             ry = (wrapn(k0y - row0 + 7, Ky, kym)) - 7;              // -7 .. H - 1
             CT val;
             if (MODE == GIN_CALLER) {
-                val = a.in[r.p];
+                val = perm_value(r.p, a.in[perm_index(r.p)]);
             } else if (MODE == GIN_SORTED) {
                 val = cx<R>(r.v.x, r.v.y);
             } else {   // GIN_PD: v = U^{1/2} d max(0, 1 - eps / rho); the item holding the window start stores it
@@ -769,12 +780,12 @@ __global__ void k_grid_merge(const GridMerge* __restrict__ merges, const Cx<R>* 
     const int ntiles = g.ntx * g.nty;
     const int l = m.tix / ntiles, t = m.tix - l * ntiles;
     const int tyi = t / g.ntx, txi = t - tyi * g.ntx;
-    CT* G = grid + (int64_t)l * g.Ky * g.Kx + (int64_t)(tyi * g.ty) * g.Kx + txi * g.tx;
+    CT* G = grid + (int64_t)l * g.Ky * g.Kw + (int64_t)(tyi * g.ty) * g.Kw + txi * g.tx;
     for (int k = threadIdx.x; k < cells; k += blockDim.x) {
         CT s = partial[(int64_t)m.slot0 * cells + k];
         for (int j = 1; j < m.nslot; ++j) s = cadd(s, partial[(int64_t)(m.slot0 + j) * cells + k]);
         const int gy = k / g.tx, gx = k - gy * g.tx;
-        G[(int64_t)gy * g.Kx + gx] = s;
+        G[(int64_t)gy * g.Kw + gx] = s;
     }
 }
 

@@ -256,19 +256,14 @@ hs_status sweep_lists(int Kx, int Ky, int L, const int64_t* off, const int* k0xs
     return HS_OK;
 }
 
-static hs_status build_sweep(Plan* p, const std::vector<int>& perm, const std::vector<int>& cellx,
-                             const std::vector<int>& celly) {
-    const int Kx = p->g.Kx, Ky = p->g.Ky;
-    const int64_t M = p->off_h[p->g.L];
-    std::vector<int> k0x(M), k0y(M);
-    for (int64_t r = 0; r < M; ++r) {
-        const int64_t i = perm[r];
-        k0x[r] = modk(cellx[i] - 3, Kx);
-        k0y[r] = modk(celly[i] - 3, Ky);
-    }
+// Grids whose strips no window reaches twice take the sweep kernel.
+static bool sweep_grid(const Plan* p) { return p->g.Kx >= 2 * GRID_TILE && p->g.Ky >= 2 * GRID_TILE; }
+
+static hs_status build_sweep(Plan* p) {
+    const int Kx = p->g.Kw, Ky = p->g.Ky;   // half plane: no window reaches the pitch, so none wraps
     std::vector<SweepItem> items;
     std::vector<int> ent;
-    HS_TRY(sweep_lists(Kx, Ky, p->g.L, p->off_h.data(), k0x.data(), k0y.data(), p->sweep_hmax, p->sweep_cap, items,
+    HS_TRY(sweep_lists(Kx, Ky, p->g.L, p->off_h.data(), p->k0x_h.data(), p->k0y_h.data(), p->sweep_hmax, p->sweep_cap, items,
                        ent));
     if (p->sw_items) {   // rebuilt by the autotuner: replace the previous lists
         plan_release(p, p->sw_items);
@@ -331,10 +326,10 @@ static hs_status time_ms(cudaStream_t s, int reps, const std::function<hs_status
     return st;
 }
 
-static hs_status autotune(Plan* p, const std::vector<int>& perm, const std::vector<int>& cellx,
-                          const std::vector<int>& celly, bool sweep, cudaStream_t s) {
+static hs_status autotune(Plan* p, cudaStream_t s) {
     const auto t0 = std::chrono::steady_clock::now();
-    const TuneKey key{p->g.Kx, p->g.Ky, p->g.L, (int)p->prec, p->flags, p->M_total};
+    const bool sweep = sweep_grid(p);
+    const TuneKey key{p->g.Kx, p->g.Ky, p->g.L, (int)p->prec, p->flags | (p->half ? 0u : 0x80000000u), p->M_total};
     {
         std::lock_guard<std::mutex> lock(g_tune_mu);
         auto it = g_tune_cache.find(key);
@@ -348,7 +343,7 @@ static hs_status autotune(Plan* p, const std::vector<int>& perm, const std::vect
             if (sweep && (v.hmax != p->sweep_hmax || v.cap != p->sweep_cap)) {
                 p->sweep_hmax = v.hmax;
                 p->sweep_cap = v.cap;
-                HS_TRY(build_sweep(p, perm, cellx, celly));
+                HS_TRY(build_sweep(p));
             }
             p->tuned = 2;
             p->tune_ms = std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t0).count();
@@ -365,7 +360,7 @@ static hs_status autotune(Plan* p, const std::vector<int>& perm, const std::vect
         for (int c = 0; c < 3; ++c) {
             p->sweep_hmax = cand[c][0];
             p->sweep_cap = cand[c][1];
-            HS_TRY(build_sweep(p, perm, cellx, celly));
+            HS_TRY(build_sweep(p));
             GridArgs a{};
             a.mode = GIN_SORTED;
             a.in = p->vis;
@@ -375,10 +370,10 @@ static hs_status autotune(Plan* p, const std::vector<int>& perm, const std::vect
         if (best != 2) {
             p->sweep_hmax = cand[best][0];
             p->sweep_cap = cand[best][1];
-            HS_TRY(build_sweep(p, perm, cellx, celly));
+            HS_TRY(build_sweep(p));
         }
     }
-    if (p->prec == HS_F32 && !(p->flags & HS_PLAN_GRAM_FMA) && L <= MAX_L_NUC) {
+    if (p->half && p->prec == HS_F32 && !(p->flags & HS_PLAN_GRAM_FMA) && L <= MAX_L_NUC) {
         HS_CHECK_CUDA(cudaMemsetAsync(p->xbuf, 0, (size_t)L * N * p->rsize(), s));
         HS_CHECK_CUDA(cudaMemsetAsync(p->xbuf2, 0, (size_t)L * N * p->rsize(), s));
         for (int c = 0; c < 2; ++c) {
@@ -411,70 +406,53 @@ static hs_status autotune(Plan* p, const std::vector<int>& perm, const std::vect
     return HS_OK;
 }
 
-static hs_status build(Plan* p, const int64_t* vis_offsets, int nblocks, const int64_t* block_offsets,
-                       const void* uv, const void* weights, const void* precond, cudaStream_t s) {
+// Everything of a plan that depends on the coverage and on the plane kept (half
+// or whole): sorted order, coordinates, work lists, tables, grid scratch.
+// uvh, wh, uh: caller order (wh, uh empty for 1).
+static hs_status build_layout(Plan* p, const std::vector<double>& uvh, const std::vector<double>& wh,
+                              const std::vector<double>& uh, cudaStream_t s) {
     Geo& g = p->g;
     const int L = g.L;
-    p->off_h.assign(vis_offsets, vis_offsets + L + 1);
-    if (p->off_h[0] != 0) return fail(HS_ERR_ARG, "vis_offsets[0] must be 0");
-    int64_t Mmax = 0;
-    for (int l = 0; l < L; ++l) {
-        const int64_t m = p->off_h[l + 1] - p->off_h[l];
-        if (m < 0) return fail(HS_ERR_ARG, "vis_offsets must be nondecreasing (channel %d)", l);
-        Mmax = std::max(Mmax, m);
-    }
-    const int64_t M = p->off_h[L];
-    if (M >= ((int64_t)1 << 31)) return fail(HS_ERR_ARG, "total visibilities must be < 2^31");
-    if (M > 0 && uv == nullptr) return fail(HS_ERR_ARG, "uv is null");
-    p->M_total = M;
-    p->Mmax = (int)Mmax;
-    // data blocks (Sec. 2.1, M_l^b): contiguous caller ranges inside channels
-    if (block_offsets == nullptr) {
-        p->blk_off_h = p->off_h;
-    } else {
-        if (nblocks < L) return fail(HS_ERR_ARG, "nblocks (%d) must be >= L (%d)", nblocks, L);
-        p->blk_off_h.assign(block_offsets, block_offsets + nblocks + 1);
-        if (p->blk_off_h[0] != 0 || p->blk_off_h[nblocks] != M)
-            return fail(HS_ERR_ARG, "block_offsets must run from 0 to the total visibility count");
-        for (int k = 0; k < nblocks; ++k)
-            if (p->blk_off_h[k + 1] < p->blk_off_h[k]) return fail(HS_ERR_ARG, "block_offsets must be nondecreasing");
-        for (int l = 1; l < L; ++l)   // every channel boundary must be a block boundary
-            if (!std::binary_search(p->blk_off_h.begin(), p->blk_off_h.end(), p->off_h[l]))
-                return fail(HS_ERR_ARG, "block_offsets must contain every channel boundary (channel %d)", l);
-    }
-    p->nblk = (int)p->blk_off_h.size() - 1;
-    p->blk_ch.assign(p->nblk, 0);
-    for (int k = 0; k < p->nblk; ++k) {   // channel of a block: the last channel starting at or before it
-        const int64_t x = p->blk_off_h[k];
-        const int l = (int)(std::upper_bound(p->off_h.begin(), p->off_h.end() - 1, x) - p->off_h.begin()) - 1;
-        p->blk_ch[k] = std::max(0, std::min(L - 1, l));
-    }
-
-    std::vector<double> uvh, wh, uh;
-    HS_TRY(download_real(p, uv, 2 * M, uvh, s));
-    if (weights) HS_TRY(download_real(p, weights, M, wh, s));
-    if (precond) HS_TRY(download_real(p, precond, M, uh, s));
-    for (int64_t i = 0; i < 2 * M; ++i) {
-        const double v = uvh[i];
-        if (!std::isfinite(v) || v < -M_PI || v >= M_PI)
-            return fail(HS_ERR_ARG, "uv[%lld] = %g outside [-pi, pi)", (long long)(i / 2), v);
-    }
-    for (int64_t i = 0; i < (int64_t)uh.size(); ++i)
-        if (!(uh[i] > 0.0) || !std::isfinite(uh[i]))
-            return fail(HS_ERR_ARG, "precond[%lld] must be finite and > 0", (long long)i);
-
+    const int64_t M = p->M_total;
+    g.Kc = p->half ? g.nx + 8 : g.Kx;
+    g.Kw = p->half ? (g.Kc + GRID_TILE - 1) / GRID_TILE * GRID_TILE : g.Kx;
+    g.kwm = pow2(g.Kw) ? g.Kw - 1 : -1;
+    g.tx = std::min(GRID_TILE, g.Kw);
+    g.ty = std::min(GRID_TILE, g.Ky);
+    g.ntx = g.Kw / g.tx;
+    g.nty = g.Ky / g.ty;
     const int Kx = g.Kx, Ky = g.Ky, TX = g.tx, TY = g.ty;
-    // per-visibility cells and fractions (FP64, same expression as t = u K / (2 pi))
+    // per-visibility cells and fractions (FP64, same expression as t = u K / (2 pi)).
+    // Half plane: samples with u < 0 are mirrored to (-u, -v): the window of -t is the mirror image of
+    // the window of t, cells floor(t) - 3 .. floor(t) + 4 reversed, also on a cell
+    // (t an integer), where the fraction of the mirrored sample is 1. cellx is the window's
+    // start column in memory (kx = floor(t) - 3: column floor(t) of the half plane, kx mod Kx
+    // of the whole one), celly the cell floor(t) mod Ky.
     std::vector<int> cellx(M), celly(M);
     std::vector<double> fx(M), fy(M);
+    std::vector<uint8_t> mirrored(M);
     for (int64_t i = 0; i < M; ++i) {
-        const double tu = uvh[2 * i] * Kx / (2.0 * M_PI);
-        const double tv = uvh[2 * i + 1] * Ky / (2.0 * M_PI);
-        const double flu = std::floor(tu), flv = std::floor(tv);
+        double tu = uvh[2 * i] * Kx / (2.0 * M_PI);
+        double tv = uvh[2 * i + 1] * Ky / (2.0 * M_PI);
+        const bool mir = p->half && tu < 0.0;
+        if (mir) {
+            tu = -tu;
+            tv = -tv;
+        }
+        double flu = std::floor(tu), flv = std::floor(tv);
         fx[i] = tu - flu;
         fy[i] = tv - flv;
-        cellx[i] = (int)((((int64_t)flu % Kx) + Kx) % Kx);
-        celly[i] = (int)((((int64_t)flv % Ky) + Ky) % Ky);
+        if (mir && fx[i] == 0.0) {
+            flu -= 1.0;
+            fx[i] = 1.0;
+        }
+        if (mir && fy[i] == 0.0) {
+            flv -= 1.0;
+            fy[i] = 1.0;
+        }
+        mirrored[i] = mir;
+        cellx[i] = p->half ? (int)flu : modk((int64_t)flu - 3, Kx);
+        celly[i] = modk((int64_t)flv, Ky);
     }
     // sort each block (each channel without blocks) by (tile of the window start, cell)
     std::vector<int> perm(M);
@@ -483,7 +461,7 @@ static hs_status build(Plan* p, const int64_t* vis_offsets, int nblocks, const i
         const int64_t a = p->blk_off_h[kb], b = p->blk_off_h[kb + 1];
         keys.resize(b - a);
         for (int64_t i = a; i < b; ++i) {
-            const int k0x = modk(cellx[i] - 3, Kx), k0y = modk(celly[i] - 3, Ky);
+            const int k0x = cellx[i], k0y = modk(celly[i] - 3, Ky);
             const uint64_t tile = (uint64_t)(k0y / TY) * g.ntx + (uint64_t)(k0x / TX);
             const uint64_t key = (tile * TY + (uint64_t)(k0y % TY)) * TX + (uint64_t)(k0x % TX);
             keys[i - a] = (key << 32) | (uint64_t)(i - a);
@@ -491,7 +469,11 @@ static hs_status build(Plan* p, const int64_t* vis_offsets, int nblocks, const i
         std::sort(keys.begin(), keys.end());
         for (int64_t r = 0; r < b - a; ++r) perm[a + r] = (int)(a + (int64_t)(keys[r] & 0xffffffffu));
     }
-    HS_TRY(upload(p, (void**)&p->perm, perm));
+    {
+        std::vector<uint32_t> pm(M);
+        for (int64_t r = 0; r < M; ++r) pm[r] = (uint32_t)perm[r] | (mirrored[perm[r]] ? PERM_MIRROR : 0u);
+        HS_TRY(upload(p, (void**)&p->perm, pm));
+    }
     if (p->nblk != L) {   // block of every sorted visibility (gridding scale lookup)
         std::vector<int> bid(M);
         for (int kb = 0; kb < p->nblk; ++kb)
@@ -513,7 +495,7 @@ static hs_status build(Plan* p, const int64_t* vis_offsets, int nblocks, const i
             while (r < b) {
                 auto tile_of = [&](int64_t rr) {
                     const int64_t i = perm[rr];
-                    const int k0x = modk(cellx[i] - 3, Kx), k0y = modk(celly[i] - 3, Ky);
+                    const int k0x = cellx[i], k0y = modk(celly[i] - 3, Ky);
                     return (int64_t)(k0y / TY) * g.ntx + k0x / TX;
                 };
                 const int64_t t = tile_of(r);
@@ -548,7 +530,7 @@ static hs_status build(Plan* p, const int64_t* vis_offsets, int nblocks, const i
             uint64_t qy = (uint64_t)std::llround(std::ldexp(fy[i], g.fby));
             if (qx >= (1ull << g.fbx)) {
                 qx = 0;
-                cxv = modk(cxv + 1, Kx);
+                cxv = p->half ? cxv + 1 : modk(cxv + 1, Kx);   // half plane: at most Kx / 2
             }
             if (qy >= (1ull << g.fby)) {
                 qy = 0;
@@ -586,17 +568,25 @@ static hs_status build(Plan* p, const int64_t* vis_offsets, int nblocks, const i
 
     // gridding lists: the sweep kernel's for grids of at least 64 x 64 cells;
     // per-tile lists for smaller grids and the compensated kernel
-    const bool sweep = Kx >= 2 * GRID_TILE && Ky >= 2 * GRID_TILE;
-    if (sweep) HS_TRY(build_sweep(p, perm, cellx, celly));
+    const bool sweep = sweep_grid(p);
+    if (sweep) {
+        p->k0x_h.resize(M);
+        p->k0y_h.resize(M);
+        for (int64_t r = 0; r < M; ++r) {
+            p->k0x_h[r] = cellx[perm[r]];
+            p->k0y_h[r] = modk(celly[perm[r]] - 3, Ky);
+        }
+        HS_TRY(build_sweep(p));
+    }
     if (!sweep || (p->flags & HS_PLAN_COMPENSATED)) {
         // gridding lists: every (channel, tile) overlapped by a window
         const int64_t nt = p->ntiles();
         std::vector<int64_t> toff((size_t)L * nt + 1, 0);
         auto tiles_of = [&](int64_t r, int* txs, int* tys, int& ntx_, int& nty_) {
             const int64_t i = perm[r];
-            const int k0x = modk(cellx[i] - 3, Kx), k0y = modk(celly[i] - 3, Ky);
+            const int k0x = cellx[i], k0y = modk(celly[i] - 3, Ky);
             txs[0] = k0x / TX;
-            txs[1] = modk(k0x + 7, Kx) / TX;
+            txs[1] = modk(k0x + 7, g.Kw) / TX;
             tys[0] = k0y / TY;
             tys[1] = modk(k0y + 7, Ky) / TY;
             ntx_ = txs[1] != txs[0] ? 2 : 1;
@@ -641,6 +631,7 @@ static hs_status build(Plan* p, const int64_t* vis_offsets, int nblocks, const i
                 d &= K - 1;
                 return d < K - d ? d : K - d;
             };
+            auto circx = [&](int d) { return p->half ? std::abs(d) : circ(d, Kx); };
             std::vector<Group> open;
             auto emit = [&](const Group& g) {
                 for (int k = 0; k < 4; ++k) gent.push_back(k < g.m ? g.e[k] : -1);
@@ -650,13 +641,13 @@ static hs_status build(Plan* p, const int64_t* vis_offsets, int nblocks, const i
                 for (int64_t q = toff[tix]; q < toff[tix + 1]; ++q) {
                     const int r = ent[q];
                     const int64_t i = perm[r];
-                    const int x = modk(cellx[i] - 3, Kx), y = modk(celly[i] - 3, Ky);
+                    const int x = cellx[i], y = modk(celly[i] - 3, Ky);
                     bool placed = false;
                     for (size_t gi = 0; gi < open.size() && !placed; ++gi) {
                         Group& g = open[gi];
                         bool fits = true;
                         for (int k = 0; k < g.m && fits; ++k)
-                            fits = circ(x - g.x[k], Kx) >= 8 || circ(y - g.y[k], Ky) >= 8;
+                            fits = circx(x - g.x[k]) >= 8 || circ(y - g.y[k], Ky) >= 8;
                         if (!fits) continue;
                         g.e[g.m] = r;
                         g.x[g.m] = x;
@@ -748,12 +739,75 @@ static hs_status build(Plan* p, const int64_t* vis_offsets, int nblocks, const i
         HS_TRY(upload_real<double>(p, &p->twy, twy));
     }
 
+    HS_TRY(plan_alloc(p, &p->grid, (size_t)L * Ky * g.Kw * p->csize()));
+    HS_TRY(plan_alloc(p, &p->tmp, (size_t)L * g.ny * g.Kc * p->csize()));
+    HS_TRY(plan_alloc(p, &p->vis, (size_t)std::max<int64_t>(M, 1) * p->csize()));
+    HS_CHECK_CUDA(cudaStreamCreateWithFlags(&p->fft_side, cudaStreamNonBlocking));
+    HS_CHECK_CUDA(cudaEventCreateWithFlags(&p->fft_ev_col, cudaEventDisableTiming));
+    HS_CHECK_CUDA(cudaEventCreateWithFlags(&p->fft_ev_join, cudaEventDisableTiming));
+    HS_TRY(fft_prepare(p));
+    if (p->flags & HS_PLAN_FFT_CHUNKED) p->fft_adj_chunk = fft_adjoint_chunk(p);
+    return HS_OK;
+}
+
+static hs_status build(Plan* p, const int64_t* vis_offsets, int nblocks, const int64_t* block_offsets,
+                       const void* uv, const void* weights, const void* precond, cudaStream_t s) {
+    Geo& g = p->g;
+    const int L = g.L;
+    p->off_h.assign(vis_offsets, vis_offsets + L + 1);
+    if (p->off_h[0] != 0) return fail(HS_ERR_ARG, "vis_offsets[0] must be 0");
+    int64_t Mmax = 0;
+    for (int l = 0; l < L; ++l) {
+        const int64_t m = p->off_h[l + 1] - p->off_h[l];
+        if (m < 0) return fail(HS_ERR_ARG, "vis_offsets must be nondecreasing (channel %d)", l);
+        Mmax = std::max(Mmax, m);
+    }
+    const int64_t M = p->off_h[L];
+    if (M >= ((int64_t)1 << 31)) return fail(HS_ERR_ARG, "total visibilities must be < 2^31");
+    if (M > 0 && uv == nullptr) return fail(HS_ERR_ARG, "uv is null");
+    p->M_total = M;
+    p->Mmax = (int)Mmax;
+    // data blocks (Sec. 2.1, M_l^b): contiguous caller ranges inside channels
+    if (block_offsets == nullptr) {
+        p->blk_off_h = p->off_h;
+    } else {
+        if (nblocks < L) return fail(HS_ERR_ARG, "nblocks (%d) must be >= L (%d)", nblocks, L);
+        p->blk_off_h.assign(block_offsets, block_offsets + nblocks + 1);
+        if (p->blk_off_h[0] != 0 || p->blk_off_h[nblocks] != M)
+            return fail(HS_ERR_ARG, "block_offsets must run from 0 to the total visibility count");
+        for (int k = 0; k < nblocks; ++k)
+            if (p->blk_off_h[k + 1] < p->blk_off_h[k]) return fail(HS_ERR_ARG, "block_offsets must be nondecreasing");
+        for (int l = 1; l < L; ++l)   // every channel boundary must be a block boundary
+            if (!std::binary_search(p->blk_off_h.begin(), p->blk_off_h.end(), p->off_h[l]))
+                return fail(HS_ERR_ARG, "block_offsets must contain every channel boundary (channel %d)", l);
+    }
+    p->nblk = (int)p->blk_off_h.size() - 1;
+    p->blk_ch.assign(p->nblk, 0);
+    for (int k = 0; k < p->nblk; ++k) {   // channel of a block: the last channel starting at or before it
+        const int64_t x = p->blk_off_h[k];
+        const int l = (int)(std::upper_bound(p->off_h.begin(), p->off_h.end() - 1, x) - p->off_h.begin()) - 1;
+        p->blk_ch[k] = std::max(0, std::min(L - 1, l));
+    }
+
+    std::vector<double> uvh, wh, uh;
+    HS_TRY(download_real(p, uv, 2 * M, uvh, s));
+    if (weights) HS_TRY(download_real(p, weights, M, wh, s));
+    if (precond) HS_TRY(download_real(p, precond, M, uh, s));
+    for (int64_t i = 0; i < 2 * M; ++i) {
+        const double v = uvh[i];
+        if (!std::isfinite(v) || v < -M_PI || v >= M_PI)
+            return fail(HS_ERR_ARG, "uv[%lld] = %g outside [-pi, pi)", (long long)(i / 2), v);
+    }
+    for (int64_t i = 0; i < (int64_t)uh.size(); ++i)
+        if (!(uh[i] > 0.0) || !std::isfinite(uh[i]))
+            return fail(HS_ERR_ARG, "precond[%lld] must be finite and > 0", (long long)i);
+
+    HS_TRY(build_layout(p, uvh, wh, uh, s));
+    if (p->prec == HS_F32 && L <= MAX_L_NUC) p->uv_h.assign(uvh.begin(), uvh.end());   // exact: FP32 inputs
+
     // scratch
     const size_t rs = p->rsize(), cs = p->csize();
     const int64_t N = p->N();
-    HS_TRY(plan_alloc(p, &p->grid, (size_t)L * Ky * Kx * cs));
-    HS_TRY(plan_alloc(p, &p->tmp, (size_t)L * g.ny * Kx * cs));
-    HS_TRY(plan_alloc(p, &p->vis, (size_t)std::max<int64_t>(M, 1) * cs));
     HS_TRY(plan_alloc(p, &p->dwt_a, (size_t)NW * L * N * rs));
     HS_TRY(plan_alloc(p, &p->dwt_b, (size_t)NW * L * N * rs));
     HS_TRY(plan_alloc(p, &p->xbuf, (size_t)L * N * rs));
@@ -767,13 +821,13 @@ static hs_status build(Plan* p, const int64_t* vis_offsets, int nblocks, const i
     HS_TRY(plan_alloc(p, (void**)&p->sv, sizeof(double) * MAX_L_NUC));
     HS_TRY(plan_alloc(p, (void**)&p->dscal, sizeof(double) * 6 * std::max(L, 1)));
     HS_TRY(plan_alloc(p, (void**)&p->err_d, sizeof(int)));
-    HS_CHECK_CUDA(cudaStreamCreateWithFlags(&p->fft_side, cudaStreamNonBlocking));
-    HS_CHECK_CUDA(cudaEventCreateWithFlags(&p->fft_ev_col, cudaEventDisableTiming));
-    HS_CHECK_CUDA(cudaEventCreateWithFlags(&p->fft_ev_join, cudaEventDisableTiming));
     HS_CHECK_CUDA(cudaMemsetAsync(p->err_d, 0, sizeof(int), s));
     if (p->flags & HS_PLAN_GRAM_FMA) p->gram_tc = 0;
-    if (p->flags & HS_PLAN_FFT_CHUNKED) p->fft_adj_chunk = fft_adjoint_chunk(p);
-    if (!(p->flags & HS_PLAN_NO_TUNE)) HS_TRY(autotune(p, perm, cellx, celly, sweep, s));
+    if (!(p->flags & HS_PLAN_NO_TUNE)) HS_TRY(autotune(p, s));
+    p->k0x_h.clear();
+    p->k0y_h.clear();
+    p->k0x_h.shrink_to_fit();
+    p->k0y_h.shrink_to_fit();
     HS_CHECK_CUDA(cudaStreamSynchronize(s));
     return HS_OK;
 }
@@ -825,18 +879,76 @@ hs_status plan_create(Plan** out, int nx, int ny, int L, const int64_t* vis_offs
     g.Ky = oversample * ny;
     g.fbx = std::min(23, 32 - ilog2(g.Kx));
     g.fby = std::min(23, 32 - ilog2(g.Ky));
-    g.kxm = pow2(g.Kx) ? g.Kx - 1 : -1;
     g.kym = pow2(g.Ky) ? g.Ky - 1 : -1;
-    g.tx = std::min(GRID_TILE, g.Kx);
-    g.ty = std::min(GRID_TILE, g.Ky);
-    g.ntx = g.Kx / g.tx;
-    g.nty = g.Ky / g.ty;
     hs_status st = build(p.get(), vis_offsets, nblocks, block_offsets, uv, weights, precond, s);
     if (st != HS_OK) {
         plan_free(p.get());
         return st;
     }
     *out = p.release();
+    return HS_OK;
+}
+
+// The whole-plane companion of an FP32 plan: same coverage, blocks, weights and
+// flags; p stays unchanged but for the shared reference.
+hs_status plane_plan(Plan* p, std::shared_ptr<Plan>* out, cudaStream_t s) {
+    std::lock_guard<std::mutex> lock(p->plane_mu);
+    *out = p->plane.lock();
+    if (*out) return HS_OK;
+    if (p->prec != HS_F32 || (int64_t)p->uv_h.size() != 2 * p->M_total)
+        return fail(HS_ERR_STATE, "whole-plane layout: the plan keeps no coverage");
+    std::shared_ptr<Plan> c(new Plan(), [](Plan* q) {
+        plan_free(q);
+        delete q;
+    });
+    c->half = false;
+    c->g = p->g;
+    c->levels = p->levels;
+    c->J = p->J;
+    c->o = p->o;
+    c->prec = p->prec;
+    c->flags = p->flags;
+    c->beta = p->beta;
+    c->M_total = p->M_total;
+    c->Mmax = p->Mmax;
+    c->off_h = p->off_h;
+    c->blk_off_h = p->blk_off_h;
+    c->blk_ch = p->blk_ch;
+    c->nblk = p->nblk;
+    const int64_t M = p->M_total;
+    std::vector<double> uvh(p->uv_h.begin(), p->uv_h.end()), wh, uh;
+    if (p->w_sorted || p->u_sorted) {   // back to caller order
+        std::vector<uint32_t> pm(M);
+        HS_CHECK_CUDA(cudaMemcpy(pm.data(), p->perm, M * sizeof(uint32_t), cudaMemcpyDeviceToHost));
+        auto unsorted = [&](const void* d, std::vector<double>& h) -> hs_status {
+            if (d == nullptr) return HS_OK;
+            std::vector<float> v(M);
+            HS_CHECK_CUDA(cudaMemcpy(v.data(), d, M * sizeof(float), cudaMemcpyDeviceToHost));
+            h.resize(M);
+            for (int64_t r = 0; r < M; ++r) h[pm[r] & ~PERM_MIRROR] = v[r];
+            return HS_OK;
+        };
+        HS_TRY(unsorted(p->w_sorted, wh));
+        HS_TRY(unsorted(p->u_sorted, uh));
+    }
+    HS_TRY(build_layout(c.get(), uvh, wh, uh, s));
+    if (!(c->flags & HS_PLAN_NO_TUNE)) {   // F^H candidates write a cube that only the tuning needs
+        const size_t bytes = (size_t)c->g.L * c->N() * c->rsize();
+        HS_TRY(lib_alloc(&c->xbuf, bytes));
+        const hs_status e = autotune(c.get(), s);
+        const cudaError_t ce = cudaStreamSynchronize(s);
+        lib_free(c->xbuf, bytes);
+        c->xbuf = nullptr;
+        HS_TRY(e);
+        HS_CHECK_CUDA(ce);
+    }
+    c->k0x_h.clear();
+    c->k0y_h.clear();
+    c->k0x_h.shrink_to_fit();
+    c->k0y_h.shrink_to_fit();
+    HS_CHECK_CUDA(cudaStreamSynchronize(s));
+    p->plane = c;
+    *out = c;
     return HS_OK;
 }
 
