@@ -19,10 +19,13 @@
 #include <atomic>
 #include <chrono>
 #include <cmath>
+#include <exception>
 #include <functional>
 #include <map>
 #include <memory>
 #include <mutex>
+#include <system_error>
+#include <thread>
 #include <tuple>
 #include <vector>
 
@@ -153,6 +156,34 @@ static hs_status download_real(const Plan* p, const void* src, int64_t n, std::v
     return HS_OK;
 }
 
+// fn(k) for k = 0 .. n - 1 on the host's cores (channels and blocks are
+// independent; results are placed by k, so they do not depend on the threads).
+// An exception of any call is thrown again here.
+static void parallel_for(int n, const std::function<void(int)>& fn) {
+    const int nt = std::min<int>(n, std::min<int>(16, std::max(1u, std::thread::hardware_concurrency())));
+    std::atomic<int> next{0};
+    std::exception_ptr err;
+    std::mutex mu;
+    auto work = [&]() {
+        for (int k; (k = next.fetch_add(1)) < n;) {
+            try {
+                fn(k);
+            } catch (...) {
+                std::lock_guard<std::mutex> lock(mu);
+                if (!err) err = std::current_exception();
+            }
+        }
+    };
+    std::vector<std::thread> ts;
+    try {
+        for (int t = 1; t < nt; ++t) ts.emplace_back(work);
+    } catch (const std::system_error&) {   // no more threads: the ones there are do the work
+    }
+    work();
+    for (auto& t : ts) t.join();
+    if (err) std::rethrow_exception(err);
+}
+
 // Gridding lists of the sweep kernel (grids of at least 64 x 64 cells). A work
 // item is one channel, one 32-column strip and its output rows [row0, row1);
 // its list holds every window that overlaps the strip and starts in rows
@@ -173,19 +204,21 @@ hs_status sweep_lists(int Kx, int Ky, int L, const int64_t* off, const int* k0xs
     struct Win {
         int y, x, r;   // start row (absolute, then relative to row0), start column relative to the strip
     };
-    std::vector<std::vector<Win>> strips(nstrip);
-    std::vector<int64_t> rowcnt(Ky);
-    std::vector<Win> seg;
-    items.clear();
-    ent.clear();
     struct Grp {
         int y, m;        // band, windows held
         uint32_t mask;   // strip columns covered
         int e[4], x[4];  // sorted visibility indices and start columns, by start column
     };
-    std::vector<Grp> open;
-    for (int l = 0; l < L; ++l) {
-        for (auto& v : strips) v.clear();
+    // channels in parallel, their lists joined in channel order
+    std::vector<std::vector<SweepItem>> ch_items(L);
+    std::vector<std::vector<int>> ch_ent(L);
+    parallel_for(L, [&](int l) {
+        std::vector<std::vector<Win>> strips(nstrip);
+        std::vector<int64_t> rowcnt(Ky);
+        std::vector<Win> seg;
+        std::vector<Grp> open;
+        std::vector<SweepItem>& items = ch_items[l];
+        std::vector<int>& ent = ch_ent[l];
         for (int64_t r = off[l]; r < off[l + 1]; ++r) {
             const int k0x = k0xs[r], k0y = k0ys[r];
             const int s0 = k0x / GRID_TILE, s1 = modk(k0x + 7, Kx) / GRID_TILE;
@@ -244,11 +277,29 @@ hs_status sweep_lists(int Kx, int Ky, int L, const int64_t* off, const int* k0xs
                     gr.mask |= mask;
                 }
                 for (const Grp& gr : open) ent.insert(ent.end(), gr.e, gr.e + 4);
-                if (ent.size() >= ((size_t)1 << 31)) return fail(HS_ERR_ARG, "too many gridding list entries");
                 items.push_back({l, st, row0, row1, e0, (int)ent.size()});
                 row0 = row1;
             }
         }
+    });
+    items.clear();
+    ent.clear();
+    size_t n_items = 0, n_ent = 0;
+    for (int l = 0; l < L; ++l) {
+        n_items += ch_items[l].size();
+        n_ent += ch_ent[l].size();
+    }
+    if (n_ent >= ((size_t)1 << 31)) return fail(HS_ERR_ARG, "too many gridding list entries");
+    items.reserve(n_items);
+    ent.reserve(n_ent);
+    for (int l = 0; l < L; ++l) {
+        const int e = (int)ent.size();
+        for (SweepItem it : ch_items[l]) {
+            it.e0 += e;
+            it.e1 += e;
+            items.push_back(it);
+        }
+        ent.insert(ent.end(), ch_ent[l].begin(), ch_ent[l].end());
     }
     std::stable_sort(items.begin(), items.end(), [](const SweepItem& a, const SweepItem& b) {
         return (a.e1 - a.e0) + 4 * (a.row1 - a.row0) > (b.e1 - b.e0) + 4 * (b.row1 - b.row0);
@@ -263,8 +314,8 @@ static hs_status build_sweep(Plan* p) {
     const int Kx = p->g.Kw, Ky = p->g.Ky;   // half plane: no window reaches the pitch, so none wraps
     std::vector<SweepItem> items;
     std::vector<int> ent;
-    HS_TRY(sweep_lists(Kx, Ky, p->g.L, p->off_h.data(), p->k0x_h.data(), p->k0y_h.data(), p->sweep_hmax, p->sweep_cap, items,
-                       ent));
+    HS_TRY(sweep_lists(Kx, Ky, p->g.L, p->off_h.data(), p->k0x_h.data(), p->k0y_h.data(), p->sweep_hmax,
+                       p->sweep_cap, items, ent));
     if (p->sw_items) {   // rebuilt by the autotuner: replace the previous lists
         plan_release(p, p->sw_items);
         plan_release(p, p->sw_ent);
@@ -431,33 +482,35 @@ static hs_status build_layout(Plan* p, const std::vector<double>& uvh, const std
     std::vector<int> cellx(M), celly(M);
     std::vector<double> fx(M), fy(M);
     std::vector<uint8_t> mirrored(M);
-    for (int64_t i = 0; i < M; ++i) {
-        double tu = uvh[2 * i] * Kx / (2.0 * M_PI);
-        double tv = uvh[2 * i + 1] * Ky / (2.0 * M_PI);
-        const bool mir = p->half && tu < 0.0;
-        if (mir) {
-            tu = -tu;
-            tv = -tv;
+    parallel_for(p->nblk, [&](int kb) {
+        for (int64_t i = p->blk_off_h[kb]; i < p->blk_off_h[kb + 1]; ++i) {
+            double tu = uvh[2 * i] * Kx / (2.0 * M_PI);
+            double tv = uvh[2 * i + 1] * Ky / (2.0 * M_PI);
+            const bool mir = p->half && tu < 0.0;
+            if (mir) {
+                tu = -tu;
+                tv = -tv;
+            }
+            double flu = std::floor(tu), flv = std::floor(tv);
+            fx[i] = tu - flu;
+            fy[i] = tv - flv;
+            if (mir && fx[i] == 0.0) {
+                flu -= 1.0;
+                fx[i] = 1.0;
+            }
+            if (mir && fy[i] == 0.0) {
+                flv -= 1.0;
+                fy[i] = 1.0;
+            }
+            mirrored[i] = mir;
+            cellx[i] = p->half ? (int)flu : modk((int64_t)flu - 3, Kx);
+            celly[i] = modk((int64_t)flv, Ky);
         }
-        double flu = std::floor(tu), flv = std::floor(tv);
-        fx[i] = tu - flu;
-        fy[i] = tv - flv;
-        if (mir && fx[i] == 0.0) {
-            flu -= 1.0;
-            fx[i] = 1.0;
-        }
-        if (mir && fy[i] == 0.0) {
-            flv -= 1.0;
-            fy[i] = 1.0;
-        }
-        mirrored[i] = mir;
-        cellx[i] = p->half ? (int)flu : modk((int64_t)flu - 3, Kx);
-        celly[i] = modk((int64_t)flv, Ky);
-    }
+    });
     // sort each block (each channel without blocks) by (tile of the window start, cell)
     std::vector<int> perm(M);
-    std::vector<uint64_t> keys;
-    for (int kb = 0; kb < p->nblk; ++kb) {
+    parallel_for(p->nblk, [&](int kb) {
+        std::vector<uint64_t> keys;
         const int64_t a = p->blk_off_h[kb], b = p->blk_off_h[kb + 1];
         keys.resize(b - a);
         for (int64_t i = a; i < b; ++i) {
@@ -468,7 +521,7 @@ static hs_status build_layout(Plan* p, const std::vector<double>& uvh, const std
         }
         std::sort(keys.begin(), keys.end());
         for (int64_t r = 0; r < b - a; ++r) perm[a + r] = (int)(a + (int64_t)(keys[r] & 0xffffffffu));
-    }
+    });
     {
         std::vector<uint32_t> pm(M);
         for (int64_t r = 0; r < M; ++r) pm[r] = (uint32_t)perm[r] | (mirrored[perm[r]] ? PERM_MIRROR : 0u);
@@ -486,9 +539,9 @@ static hs_status build_layout(Plan* p, const std::vector<double>& uvh, const std
     {
         std::vector<int> items;
         const int nb = p->nblk;
-        std::vector<int> per_b(nb, 0);
+        std::vector<std::vector<int>> b_items(nb);
         const int64_t ntl = (int64_t)g.ntx * g.nty;
-        for (int kb = 0; kb < nb; ++kb) {
+        parallel_for(nb, [&](int kb) {
             const int l = p->blk_ch[kb];
             const int64_t a = p->blk_off_h[kb], b = p->blk_off_h[kb + 1];
             int64_t r = a;
@@ -503,14 +556,16 @@ static hs_status build_layout(Plan* p, const std::vector<double>& uvh, const std
                 while (e < b && tile_of(e) == t) ++e;
                 for (int64_t c0 = r; c0 < e; c0 += DEGRID_CHUNK) {
                     const int64_t c1 = std::min<int64_t>(e, c0 + DEGRID_CHUNK);
-                    items.insert(items.end(), {(int)(l * ntl + t), (int)c0, (int)c1, kb});
-                    ++per_b[kb];
+                    b_items[kb].insert(b_items[kb].end(), {(int)(l * ntl + t), (int)c0, (int)c1, kb});
                 }
                 r = e;
             }
-        }
+        });
         int mx = 1;
-        for (int kb = 0; kb < nb; ++kb) mx = std::max(mx, per_b[kb]);
+        for (int kb = 0; kb < nb; ++kb) {
+            mx = std::max(mx, (int)(b_items[kb].size() / 4));
+            items.insert(items.end(), b_items[kb].begin(), b_items[kb].end());
+        }
         std::vector<int> seen(nb, 0);
         for (size_t k = 0; k < items.size(); k += 4) {   // slot = block * items_max + rank in block
             const int kb = items[k + 3];
@@ -523,24 +578,26 @@ static hs_status build_layout(Plan* p, const std::vector<double>& uvh, const std
 
     if (p->prec == HS_F32) {
         std::vector<uint32_t> c((size_t)2 * M);
-        for (int64_t r = 0; r < M; ++r) {
-            const int64_t i = perm[r];
-            int cxv = cellx[i], cyv = celly[i];
-            uint64_t qx = (uint64_t)std::llround(std::ldexp(fx[i], g.fbx));
-            uint64_t qy = (uint64_t)std::llround(std::ldexp(fy[i], g.fby));
-            if (qx >= (1ull << g.fbx)) {
-                qx = 0;
-                cxv = p->half ? cxv + 1 : modk(cxv + 1, Kx);   // half plane: at most Kx / 2
+        parallel_for(p->nblk, [&](int kb) {
+        for     (int64_t r = p->blk_off_h[kb]; r < p->blk_off_h[kb + 1]; ++r) {
+                const int64_t i = perm[r];
+                int cxv = cellx[i], cyv = celly[i];
+                uint64_t qx = (uint64_t)std::llround(std::ldexp(fx[i], g.fbx));
+                uint64_t qy = (uint64_t)std::llround(std::ldexp(fy[i], g.fby));
+                if (qx >= (1ull << g.fbx)) {
+                    qx = 0;
+                    cxv = p->half ? cxv + 1 : modk(cxv + 1, Kx);   // half plane: at most Kx / 2
+                }
+                if (qy >= (1ull << g.fby)) {
+                    qy = 0;
+                    cyv = modk(cyv + 1, Ky);
+                }
+                c[2 * r] = ((uint32_t)cxv << g.fbx) | (uint32_t)qx;
+                c[2 * r + 1] = ((uint32_t)cyv << g.fby) | (uint32_t)qy;
+                cellx[i] = cxv;   // tile membership below uses the stored cell
+                celly[i] = cyv;
             }
-            if (qy >= (1ull << g.fby)) {
-                qy = 0;
-                cyv = modk(cyv + 1, Ky);
-            }
-            c[2 * r] = ((uint32_t)cxv << g.fbx) | (uint32_t)qx;
-            c[2 * r + 1] = ((uint32_t)cyv << g.fby) | (uint32_t)qy;
-            cellx[i] = cxv;   // tile membership below uses the stored cell
-            celly[i] = cyv;
-        }
+        });
         HS_TRY(upload(p, &p->coords, c));
     } else {
         std::vector<Coord64> c(M);
