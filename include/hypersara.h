@@ -81,7 +81,8 @@ typedef enum { HS_F32 = 0, HS_F64 = 1 } hs_prec;
 #define HS_PLAN_GRAM_FMA 2u
 /* Keep the default parameters instead of timing candidates at creation. By
  * default a plan times, on itself, the sweep-gridding row cut and list cap
- * ((32, 512), (64, 1024), (128, 2048)), F^H over all channels at once against
+ * ((32, 512), (64, 1024), (128, 2048), and forms with 4 or 8 warps to a work
+ * item, which are not reported), F^H over all channels at once against
  * L2-sized channel chunks and, for FP32 plans, the tensor-core against the
  * CUDA-core Gram matrix, and keeps the fastest (choices cached per
  * process by grid, L, visibilities, precision and flags; hs_plan_info reports

@@ -160,6 +160,9 @@ struct Plan {
     int gram_tc = 1;                   // FP32 Gram matrix on the tensor cores (else CUDA cores)
     int sweep_hmax = SWEEP_HMAX;       // sweep gridding: most output rows per work item
     int sweep_cap = SWEEP_CAP;         // ... windows above which an item's rows are cut short
+    int sw_rows = SWEEP_HMAX;          // the lists' own row cut and cap: those above, or
+    int sw_cap = SWEEP_CAP;            // ... a form with sw_coop warps to an item
+    int sw_coop = 0;                   // warps sharing an item (0: one warp per item)
     int fft_adj_chunk = 0;             // channels per F^H chunk (0: all at once)
     int tuned = 0;                     // 1: timed at creation, 2: taken from the process cache
     double tune_ms = 0.0;              // host time spent tuning

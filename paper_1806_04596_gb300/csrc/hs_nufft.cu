@@ -566,6 +566,7 @@ __global__ void __launch_bounds__(GRID_PW * 32) k_grid_groups(NufftK<R> a, const
 // next batch's list entries and inputs are loaded before the current batch's
 // groups are added.
 constexpr int SW_WARPS = 4;      // warps (work items) per CTA
+constexpr int SW_COOP_MAX = 8;   // most warps sharing an item
 
 // 4 consecutive reals from 16-byte aligned shared memory
 __device__ __forceinline__ void sw_ld4(const float* p, float* v) {
@@ -584,30 +585,47 @@ template <typename R> struct SwRaw {
     int p;                  // caller index (GIN_CALLER) or data block (GIN_PD with blocks)
 };
 
-template <typename R, int NC, int MODE>
-__global__ void __launch_bounds__(SW_WARPS * 32, sizeof(R) == 4 ? 5 : 1)
+// Shared memory of one warp of the sweep.
+template <typename R> struct alignas(16) SwWarp {
+    // row taps of every slot, placed at their rows; with 12 reals per slot the 4
+    // slots of a group fall in disjoint banks for 16-byte loads
+    R rowt[32][12];
+    // per group and strip column: column tap x value, and 4 x batch + slot in the
+    // group (rows padded to 33 entries: the decode's scattered stores of different
+    // groups fall in different banks)
+    typename CxT<R>::T coltv[8][33];
+    int coltg[8][33];
+    int sjb[8];   // band of every group
+};
+
+// COOP: the warps of a CTA share one item. Warp w takes batches w, w + n, ... of its
+// list into banks of its own, stores its rows to shared memory, and the CTA adds the
+// copies in warp order. A dense strip cannot be cut finer by rows (one output row
+// needs the windows of 8), so where a plan has few items for the chip the longest
+// item is what a launch waits for. us per launch, one warp per item -> shared: FP64
+// 64 x 64, L = 4, 2000 per channel 350 -> 168 (8 warps, 16 rows), FP32 the same 38 -> 17,
+// FP32 256 x 256, L = 8 40 -> 25 (8, 32 rows), 640 x 384, L = 7 44 -> 41 (4, 32 rows);
+// 256 x 256, L = 60 123 -> 163, so the autotuner decides by timing.
+template <typename R, int NC, int MODE, bool COOP>
+__global__ void __launch_bounds__(COOP ? SW_COOP_MAX * 32 : SW_WARPS * 32, sizeof(R) == 4 ? (COOP ? 2 : 5) : 1)
     k_grid_sweep(const NufftK<R> a, const SweepItem* __restrict__ items,
                  const int* __restrict__ ent, int n_items) {
     typedef Cx<R> CT;
     constexpr int NE = (NC + 1) / 2, NO = NC / 2;   // even / odd coefficients of a piece
-    // row taps of every slot, placed at their rows; with 12 reals per slot the 4
-    // slots of a group fall in disjoint banks for 16-byte loads
-    constexpr int RLD = 12;
-    __shared__ __align__(16) R rowt[SW_WARPS][32][RLD];
-    // per group and strip column: column tap x value, and 4 x batch + slot in the
-    // group (rows padded to 33 entries: the decode's scattered stores of different
-    // groups fall in different banks)
-    __shared__ __align__(16) CT coltv[SW_WARPS][8][33];
-    __shared__ int coltg[SW_WARPS][8][33];
-    __shared__ int sjb[SW_WARPS][8];                          // band of every group
+    extern __shared__ __align__(16) unsigned char smem_raw[];
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int wi = blockIdx.x * SW_WARPS + w;
+    const int nw = blockDim.x >> 5;
+    SwWarp<R>& sw = reinterpret_cast<SwWarp<R>*>(smem_raw)[w];
+    const int wi = COOP ? blockIdx.x : blockIdx.x * SW_WARPS + w;
     if (wi >= n_items) return;
+    const int step = COOP ? 32 * nw : 32;   // slots between a warp's batches
     const SweepItem it = items[wi];
     const int Kw = a.g.Kw, Ky = a.g.Ky;
     const int kwm = a.g.kwm, kym = a.g.kym;
     const int c0 = it.strip * GRID_TILE, row0 = it.row0, H = it.row1 - it.row0;
     CT* out = a.grid_out + (int64_t)it.l * Ky * Kw + (int64_t)row0 * Kw + c0 + lane;
+    CT* copies = reinterpret_cast<CT*>(reinterpret_cast<SwWarp<R>*>(smem_raw) + nw);   // COOP: [nw][H][32]
+    CT* own = copies + (int64_t)w * H * 32 + lane;
     CT B0[4], B1[4], B2[4];
 #pragma unroll
     for (int k = 0; k < 4; ++k) B0[k] = B1[k] = B2[k] = cx<R>(0, 0);
@@ -652,7 +670,10 @@ __global__ void __launch_bounds__(SW_WARPS * 32, sizeof(R) == 4 ? 5 : 1)
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
             const int r = 4 * jb + k;
-            if ((unsigned)r < (unsigned)H) out[(int64_t)r * Kw] = U[k];
+            if ((unsigned)r < (unsigned)H) {
+                if (COOP) own[r * 32] = U[k];
+                else out[(int64_t)r * Kw] = U[k];
+            }
             U[k] = cx<R>(0, 0);
         }
     };
@@ -675,24 +696,25 @@ __global__ void __launch_bounds__(SW_WARPS * 32, sizeof(R) == 4 ? 5 : 1)
         }
     };
 
-    int i_cur = it.e0 + lane < it.e1 ? ent[it.e0 + lane] : -1;
+    const int first = it.e0 + (COOP ? 32 * w : 0);
+    int i_cur = first + lane < it.e1 ? ent[first + lane] : -1;
     SwRaw<R> r_cur;
     load_raw(i_cur, r_cur);
-    int i_nxt = it.e0 + 32 + lane < it.e1 ? ent[it.e0 + 32 + lane] : -1;
-    R* rt = rowt[w][lane];
+    int i_nxt = first + step + lane < it.e1 ? ent[first + step + lane] : -1;
+    R* rt = sw.rowt[lane];
     for (int k = lane; k < 8 * 33; k += 32) {
-        (&coltv[w][0][0])[k] = cx<R>(0, 0);
-        (&coltg[w][0][0])[k] = -1;
+        (&sw.coltv[0][0])[k] = cx<R>(0, 0);
+        (&sw.coltg[0][0])[k] = -1;
     }
     __syncwarp();
     int nbat = 0;   // batch number (tag of the column entries written by this batch)
-    for (int b0 = it.e0; b0 < it.e1; b0 += 32) {
+    for (int b0 = first; b0 < it.e1; b0 += step) {
         // ---- decode slot b0 + lane
         const int i = i_cur;
         const SwRaw<R> r = r_cur;
         i_cur = i_nxt;
         load_raw(i_cur, r_cur);   // next batch's inputs (their entries were loaded a batch ago)
-        i_nxt = b0 + 64 + lane < it.e1 ? ent[b0 + 64 + lane] : -1;
+        i_nxt = b0 + 2 * step + lane < it.e1 ? ent[b0 + 2 * step + lane] : -1;
         int ry = 0;
         if (i >= 0) {
             int cxv, cyv;
@@ -728,32 +750,32 @@ __global__ void __launch_bounds__(SW_WARPS * 32, sizeof(R) == 4 ? 5 : 1)
                 const int c = rx + m;
                 if ((unsigned)c < 32u)
                 {
-                    coltv[w][g][c] = cx<R>(pu[m] * val.x, pu[m] * val.y);
-                    coltg[w][g][c] = (nbat << 2) | (lane & 3);
+                    sw.coltv[g][c] = cx<R>(pu[m] * val.x, pu[m] * val.y);
+                    sw.coltg[g][c] = (nbat << 2) | (lane & 3);
                 }
             }
         }
-        if ((lane & 3) == 0) sjb[w][lane >> 2] = ry >> 2;
+        if ((lane & 3) == 0) sw.sjb[lane >> 2] = ry >> 2;
         __syncwarp();
         // ---- add the batch's groups
         // (each group's column entry and band are read one group ahead)
         const int ng = min(8, (it.e1 - b0) >> 2);
-        CT cv_n = coltv[w][0][lane];
-        int cg_n = coltg[w][0][lane];
-        int gj_n = sjb[w][0];
+        CT cv_n = sw.coltv[0][lane];
+        int cg_n = sw.coltg[0][lane];
+        int gj_n = sw.sjb[0];
         for (int q = 0; q < ng; ++q) {
             const CT cv = cv_n;
             const int cg = cg_n;
             const int gj = gj_n;
             const bool cur = (cg >> 2) == nbat;
-            const R* pvs = rowt[w][4 * q + (cur ? (cg & 3) : 0)];
+            const R* pvs = sw.rowt[4 * q + (cur ? (cg & 3) : 0)];
             R pv[12];
 #pragma unroll
             for (int k = 0; k < 12; k += 4) sw_ld4(pvs + k, pv + k);
             const int qn = min(q + 1, 7);
-            cv_n = coltv[w][qn][lane];
-            cg_n = coltg[w][qn][lane];
-            gj_n = sjb[w][qn];
+            cv_n = sw.coltv[qn][lane];
+            cg_n = sw.coltg[qn][lane];
+            gj_n = sw.sjb[qn];
             while (jb < gj) advance();
             const CT t = cur ? cv : cx<R>(0, 0);
             if (jm == 0) add(B0, B1, B2, pv, t);
@@ -764,6 +786,14 @@ __global__ void __launch_bounds__(SW_WARPS * 32, sizeof(R) == 4 ? 5 : 1)
         ++nbat;
     }
     while (4 * jb < H) advance();
+    if constexpr (COOP) {
+        __syncthreads();
+        for (int k = threadIdx.x; k < H * 32; k += blockDim.x) {
+            CT v = copies[k];
+            for (int q = 1; q < nw; ++q) v = cadd(v, copies[q * H * 32 + k]);
+            out[(int64_t)(k >> 5) * Kw] = v;   // (k & 31) = lane
+        }
+    }
 }
 
 // Sum of the partial tiles of every split tile (fixed slot order).
@@ -851,9 +881,15 @@ template <typename R, int NC, int MODE, bool KAHAN>
 static hs_status grid_launch(Plan* p, NufftK<R>& k, cudaStream_t s) {
     const size_t smem = (size_t)GRID_WARPS * p->g.tx * p->g.ty * sizeof(Cx<R>) * (KAHAN ? 2 : 1);
     if (!KAHAN && p->n_sw_items > 0) {
-        const unsigned nb = (unsigned)((p->n_sw_items + SW_WARPS - 1) / SW_WARPS);
-        k_grid_sweep<R, NC, MODE><<<nb, SW_WARPS * 32, 0, s>>>(k, (const SweepItem*)p->sw_items, p->sw_ent,
-                                                             (int)p->n_sw_items);
+        const SweepItem* it = (const SweepItem*)p->sw_items;
+        const int n = (int)p->n_sw_items;
+        if (p->sw_coop > 0) {
+            const size_t sm = p->sw_coop * (sizeof(SwWarp<R>) + (size_t)p->sw_rows * 32 * sizeof(Cx<R>));
+            k_grid_sweep<R, NC, MODE, true><<<n, p->sw_coop * 32, sm, s>>>(k, it, p->sw_ent, n);
+        } else {
+            k_grid_sweep<R, NC, MODE, false><<<(n + SW_WARPS - 1) / SW_WARPS, SW_WARPS * 32,
+                                               SW_WARPS * sizeof(SwWarp<R>), s>>>(k, it, p->sw_ent, n);
+        }
         HS_CHECK_LAUNCH();
         return HS_OK;
     }
@@ -880,9 +916,12 @@ template <typename R, int NC, int MODE, bool KAHAN> static hs_status grid_attr()
     static_assert(sizeof(GridItem) == 16 && sizeof(GridMerge) == 12, "plan-side layout");
     HS_CHECK_CUDA(cudaFuncSetAttribute(k_grid<R, NC, MODE, KAHAN>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-    if (!KAHAN)
+    if constexpr (!KAHAN) {
+        HS_CHECK_CUDA(cudaFuncSetAttribute(k_grid_sweep<R, NC, MODE, true>,
+                                           cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024));
         HS_CHECK_CUDA(cudaFuncSetAttribute(k_grid_groups<R, NC, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                            (int)(GRID_PW * GRID_TILE * GRID_LDT * sizeof(Cx<R>))));
+    }
     return HS_OK;
 }
 

@@ -158,9 +158,12 @@ static hs_status download_real(const Plan* p, const void* src, int64_t n, std::v
 
 // fn(k) for k = 0 .. n - 1 on the host's cores (channels and blocks are
 // independent; results are placed by k, so they do not depend on the threads).
+// items: visibilities in all; one more thread per 32 768 (below that, starting
+// threads costs more than it gains: 60 channels of 16 took 5.7 instead of 2.5 ms).
 // An exception of any call is thrown again here.
-static void parallel_for(int n, const std::function<void(int)>& fn) {
-    const int nt = std::min<int>(n, std::min<int>(16, std::max(1u, std::thread::hardware_concurrency())));
+static void parallel_for(int n, int64_t items, const std::function<void(int)>& fn) {
+    const int64_t most = std::min<int64_t>(std::max(1u, std::thread::hardware_concurrency()), 1 + items / 32768);
+    const int nt = (int)std::min<int64_t>(n, std::min<int64_t>(16, most));
     std::atomic<int> next{0};
     std::exception_ptr err;
     std::mutex mu;
@@ -212,7 +215,7 @@ hs_status sweep_lists(int Kx, int Ky, int L, const int64_t* off, const int* k0xs
     // channels in parallel, their lists joined in channel order
     std::vector<std::vector<SweepItem>> ch_items(L);
     std::vector<std::vector<int>> ch_ent(L);
-    parallel_for(L, [&](int l) {
+    parallel_for(L, off[L], [&](int l) {
         std::vector<std::vector<Win>> strips(nstrip);
         std::vector<int64_t> rowcnt(Ky);
         std::vector<Win> seg;
@@ -314,8 +317,8 @@ static hs_status build_sweep(Plan* p) {
     const int Kx = p->g.Kw, Ky = p->g.Ky;   // half plane: no window reaches the pitch, so none wraps
     std::vector<SweepItem> items;
     std::vector<int> ent;
-    HS_TRY(sweep_lists(Kx, Ky, p->g.L, p->off_h.data(), p->k0x_h.data(), p->k0y_h.data(), p->sweep_hmax,
-                       p->sweep_cap, items, ent));
+    HS_TRY(sweep_lists(Kx, Ky, p->g.L, p->off_h.data(), p->k0x_h.data(), p->k0y_h.data(), p->sw_rows,
+                       p->sw_cap, items, ent));
     if (p->sw_items) {   // rebuilt by the autotuner: replace the previous lists
         plan_release(p, p->sw_items);
         plan_release(p, p->sw_ent);
@@ -334,7 +337,8 @@ static hs_status build_sweep(Plan* p) {
 // sampling density, by timing the candidates on this plan with CUDA events
 // (inputs: zeroed plan scratch; the values do not change the work):
 //   * sweep gridding row cut and list cap, (32, 512), (64, 1024), (128, 2048):
-//     short items balance dense coverage, tall items cut the halo rows;
+//     short items balance dense coverage, tall items cut the halo rows; on the half plane also
+//     4 or 8 warps to an item (64, 32 or 16 rows), for plans with few items;
 //   * FP32 Gram matrix of the nuclear prox on the tensor cores or the CUDA
 //     cores (the tensor-core form streams 64-pixel chunks per SM and wins on
 //     large cubes; the CUDA-core form wins when N L is small);
@@ -352,7 +356,7 @@ struct TuneKey {
     }
 };
 struct TuneVal {
-    int gram_tc, hmax, cap, fft_chunk;
+    int gram_tc, hmax, cap, rows, rcap, coop, fft_chunk;
     double grid_ms[3], gram_ms[2], fft_ms[2];
 };
 std::mutex g_tune_mu;
@@ -391,9 +395,12 @@ static hs_status autotune(Plan* p, cudaStream_t s) {
             std::copy(v.grid_ms, v.grid_ms + 3, p->tune_grid_ms);
             std::copy(v.gram_ms, v.gram_ms + 2, p->tune_gram_ms);
             std::copy(v.fft_ms, v.fft_ms + 2, p->tune_fft_ms);
-            if (sweep && (v.hmax != p->sweep_hmax || v.cap != p->sweep_cap)) {
-                p->sweep_hmax = v.hmax;
-                p->sweep_cap = v.cap;
+            p->sweep_hmax = v.hmax;
+            p->sweep_cap = v.cap;
+            p->sw_coop = v.coop;
+            if (sweep && (v.rows != p->sw_rows || v.rcap != p->sw_cap)) {
+                p->sw_rows = v.rows;
+                p->sw_cap = v.rcap;
                 HS_TRY(build_sweep(p));
             }
             p->tuned = 2;
@@ -408,19 +415,41 @@ static hs_status autotune(Plan* p, cudaStream_t s) {
         static const int cand[3][2] = {{32, 512}, {64, 1024}, {128, 2048}};
         HS_CHECK_CUDA(cudaMemsetAsync(p->vis, 0, (size_t)p->M_total * p->csize(), s));
         int best = -1;
-        for (int c = 0; c < 3; ++c) {
-            p->sweep_hmax = cand[c][0];
-            p->sweep_cap = cand[c][1];
+        auto time_lists = [&](int rows, int cap, int coop, double* ms) -> hs_status {
+            p->sw_rows = rows;
+            p->sw_cap = cap;
+            p->sw_coop = coop;
             HS_TRY(build_sweep(p));
             GridArgs a{};
             a.mode = GIN_SORTED;
             a.in = p->vis;
-            HS_TRY(time_ms(s, reps, [&]() { return grid(p, a, s); }, &p->tune_grid_ms[c]));
+            return time_ms(s, reps, [&]() { return grid(p, a, s); }, ms);
+        };
+        for (int c = 0; c < 3; ++c) {
+            HS_TRY(time_lists(cand[c][0], cand[c][1], 0, &p->tune_grid_ms[c]));
             if (best < 0 || p->tune_grid_ms[c] < p->tune_grid_ms[best]) best = c;
         }
-        if (best != 2) {
-            p->sweep_hmax = cand[best][0];
-            p->sweep_cap = cand[best][1];
+        p->sweep_hmax = cand[best][0];
+        p->sweep_cap = cand[best][1];
+        int form[3] = {p->sweep_hmax, p->sweep_cap, 0};
+        if (p->half) {   // several warps to an item: kept when it gains more than 3 %
+            static const int shared[4][2] = {{64, 4}, {32, 4}, {32, 8}, {16, 8}};   // rows, warps
+            double t = 0.97 * p->tune_grid_ms[best];
+            for (const auto& q : shared) {
+                double ms = 0.0;
+                HS_TRY(time_lists(q[0], SWEEP_CAP * q[1], q[1], &ms));
+                if (ms < t) {
+                    t = ms;
+                    form[0] = q[0];
+                    form[1] = SWEEP_CAP * q[1];
+                    form[2] = q[1];
+                }
+            }
+        }
+        p->sw_coop = form[2];
+        if (p->sw_rows != form[0] || p->sw_cap != form[1]) {
+            p->sw_rows = form[0];
+            p->sw_cap = form[1];
             HS_TRY(build_sweep(p));
         }
     }
@@ -446,7 +475,7 @@ static hs_status autotune(Plan* p, cudaStream_t s) {
     HS_CHECK_CUDA(cudaStreamSynchronize(s));
     {
         std::lock_guard<std::mutex> lock(g_tune_mu);
-        TuneVal v{p->gram_tc, p->sweep_hmax, p->sweep_cap, p->fft_adj_chunk, {}, {}, {}};
+        TuneVal v{p->gram_tc, p->sweep_hmax, p->sweep_cap, p->sw_rows, p->sw_cap, p->sw_coop, p->fft_adj_chunk, {}, {}, {}};
         std::copy(p->tune_grid_ms, p->tune_grid_ms + 3, v.grid_ms);
         std::copy(p->tune_gram_ms, p->tune_gram_ms + 2, v.gram_ms);
         std::copy(p->tune_fft_ms, p->tune_fft_ms + 2, v.fft_ms);
@@ -482,7 +511,7 @@ static hs_status build_layout(Plan* p, const std::vector<double>& uvh, const std
     std::vector<int> cellx(M), celly(M);
     std::vector<double> fx(M), fy(M);
     std::vector<uint8_t> mirrored(M);
-    parallel_for(p->nblk, [&](int kb) {
+    parallel_for(p->nblk, M, [&](int kb) {
         for (int64_t i = p->blk_off_h[kb]; i < p->blk_off_h[kb + 1]; ++i) {
             double tu = uvh[2 * i] * Kx / (2.0 * M_PI);
             double tv = uvh[2 * i + 1] * Ky / (2.0 * M_PI);
@@ -509,7 +538,7 @@ static hs_status build_layout(Plan* p, const std::vector<double>& uvh, const std
     });
     // sort each block (each channel without blocks) by (tile of the window start, cell)
     std::vector<int> perm(M);
-    parallel_for(p->nblk, [&](int kb) {
+    parallel_for(p->nblk, M, [&](int kb) {
         std::vector<uint64_t> keys;
         const int64_t a = p->blk_off_h[kb], b = p->blk_off_h[kb + 1];
         keys.resize(b - a);
@@ -541,7 +570,7 @@ static hs_status build_layout(Plan* p, const std::vector<double>& uvh, const std
         const int nb = p->nblk;
         std::vector<std::vector<int>> b_items(nb);
         const int64_t ntl = (int64_t)g.ntx * g.nty;
-        parallel_for(nb, [&](int kb) {
+        parallel_for(nb, M, [&](int kb) {
             const int l = p->blk_ch[kb];
             const int64_t a = p->blk_off_h[kb], b = p->blk_off_h[kb + 1];
             int64_t r = a;
@@ -578,7 +607,7 @@ static hs_status build_layout(Plan* p, const std::vector<double>& uvh, const std
 
     if (p->prec == HS_F32) {
         std::vector<uint32_t> c((size_t)2 * M);
-        parallel_for(p->nblk, [&](int kb) {
+        parallel_for(p->nblk, M, [&](int kb) {
         for     (int64_t r = p->blk_off_h[kb]; r < p->blk_off_h[kb + 1]; ++r) {
                 const int64_t i = perm[r];
                 int cxv = cellx[i], cyv = celly[i];

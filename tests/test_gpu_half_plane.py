@@ -51,3 +51,22 @@ def test_edges_of_the_half_plane_match_the_oracle(cuda_device, nx, ny, prec, com
     op = oracle_op(c)
     assert_close(host(plan.phi_fwd(dev(c["X"], prec))), op.forward(c["X"]), prec)
     assert_close(host(plan.phi_adj(dev(c["Y"], prec, True))), op.adjoint(c["Y"]), prec)
+
+
+@pytest.mark.parametrize("prec", ["f64", "f32"])
+@pytest.mark.parametrize("nx,ny,M", [(32, 32, 1), (32, 96, 33), (64, 64, 4000), (96, 64, 2500), (64, 320, 3000)])
+def test_shared_gridding_items_match_the_oracle(cuda_device, nx, ny, M, prec):
+    """Few, dense work items, where the tuner takes the form with several warps to
+    an item: one window, one batch and a bit, and thousands of windows packed into a
+    few rows around the origin (so that every warp of an item holds a share)."""
+    import __graft_entry__ as ge
+    ge.build()
+    from paper_1806_04596_gb300 import hypersara as hs
+    rng = np.random.Generator(np.random.PCG64(1000 * nx + ny + M))
+    uv = rng.normal(0.0, [16.0 * np.pi / nx, 10.0 * np.pi / ny], (2 * M, 2))
+    uv = np.clip(uv, -3.0, 3.0)
+    c = dict(nx=nx, ny=ny, L=2, off=np.array([0, M, 2 * M], dtype=np.int64), uv=uv, X=np.zeros((2, ny, nx)),
+             Y=rng.standard_normal(2 * M) + 1j * rng.standard_normal(2 * M), rng=rng)
+    c = rounded(c, prec)
+    plan = hs.Plan(nx, ny, c["off"], dev(c["uv"], prec), levels=1, prec=prec)
+    assert_close(host(plan.phi_adj(dev(c["Y"], prec, True))), oracle_op(c).adjoint(c["Y"]), prec)
