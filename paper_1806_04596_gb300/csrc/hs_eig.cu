@@ -24,6 +24,7 @@
 //  3. Cholesky QR keeps the active vectors orthonormal in FP64.
 //  4. The factor is returned in low-rank form: M = I - sum_active (1 - f) x x^T
 //     (dual) or sum_active f x x^T (prox), as r, g and the active x.
+#include <algorithm>
 #include <cmath>
 
 #include "hs_device.cuh"
@@ -56,18 +57,29 @@ __device__ void rr_schedule(int n, unsigned short* pairs) {
 
 // Rotation (c, s) that zeroes a_pq of the 2 x 2 block [[a_pp, a_pq], [a_pq, a_qq]]
 // (Golub & Van Loan Alg. 8.4.1). FP32: fast reciprocal and reciprocal square
-// root (the FP32 sweeps only need FP32-orthogonal rotations); FP64: IEEE.
+// root (the FP32 sweeps only need FP32-orthogonal rotations).
 __device__ __forceinline__ void jac_rot(float app, float aqq, float apq, float& c, float& s) {
     const float tau = __fdividef(aqq - app, 2.f * apq);
     const float t = copysignf(1.f, tau) * __frcp_rn(fabsf(tau) + sqrtf(fmaf(tau, tau, 1.f)));
     c = rsqrtf(fmaf(t, t, 1.f));
     s = t * c;
 }
+// FP64: the division and the roots of the library cost ~20 dependent FP64 instructions
+// each at 1/64 of the FP32 rate, and a round waits for them. The tangent is taken to
+// FP32 accuracy (a rotation then leaves ~1e-7 of a_pq, which later rounds remove);
+// what has to be FP64 is c^2 + s^2 = 1: c = (1 + t^2)^-1/2 by two Newton steps.
 __device__ __forceinline__ void jac_rot(double app, double aqq, double apq, double& c, double& s) {
-    const double tau = (aqq - app) / (2.0 * apq);
-    const double t = copysign(1.0, tau) / (fabs(tau) + sqrt(fma(tau, tau, 1.0)));
-    c = rsqrt(fma(t, t, 1.0));
-    s = t * c;
+    double r;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(2.0 * apq));
+    float tau = (float)((aqq - app) * r);
+    if (isnan(tau)) tau = 0.f;   // equal diagonal over a subnormal a_pq
+    const double t = (double)copysignf(__frcp_rn(fabsf(tau) + sqrtf(fmaf(tau, tau, 1.f))), tau);
+    const double u = fma(t, t, 1.0);
+    double y = (double)rsqrtf((float)u);
+    y = fma(0.5 * y, fma(-(u * y), y, 1.0), y);
+    y = fma(0.5 * y, fma(-(u * y), y, 1.0), y);
+    c = y;
+    s = t * y;
 }
 
 // Cyclic Jacobi, round-robin parallel ordering, on the symmetric N x N matrix
@@ -140,7 +152,7 @@ __device__ void jacobi_blocks(T* A, T* V, unsigned short* pairs, double skip, do
                 const T r1x = si * a00 + ci * a10, r1y = si * a01 + ci * a11;
                 T b00 = cj * r0x - sj * r0y, b01 = sj * r0x + cj * r0y;
                 T b10 = cj * r1x - sj * r1y, b11 = sj * r1x + cj * r1y;
-                if (bi == bj && si != T(0)) {   // the rotated pair is decoupled
+                if (sizeof(T) == 4 && bi == bj && si != T(0)) {   // FP32: the rotated pair is decoupled
                     b01 = T(0);
                     b10 = T(0);
                 }
@@ -521,7 +533,12 @@ __global__ void __launch_bounds__(EIG_T) k_eig_f64(const double* __restrict__ Sg
 hs_status eig_f64_launch(const double* S, int L, const double* w_sv, double thr, int dual, double* Mf,
                          double* sv_out, int* r_out, cudaStream_t s) {
     const size_t sm = (size_t)4 * MAX_L_NUC * LD32 * sizeof(double);
-    k_eig_f64<<<1, EIG_T, sm, s>>>(S, L, w_sv, thr, dual, Mf, sv_out, r_out);
+    // as many threads as a round has 2 x 2 blocks (n^2 / 4, n the padded size): small matrices
+    // are bound by the barriers and block sums of a round (L = 6: one warp instead of 32)
+    int n = 2;
+    while (n < L) n <<= 1;
+    const int threads = std::max(n * n / 4, 64) > EIG_T ? EIG_T : std::max(n * n / 4, 64);
+    k_eig_f64<<<1, threads, sm, s>>>(S, L, w_sv, thr, dual, Mf, sv_out, r_out);
     HS_CHECK_LAUNCH();
     return HS_OK;
 }
