@@ -245,6 +245,14 @@ HS_API hs_status hs_prox_l21(hs_plan_t plan, const void* A, const void* w_rows, 
 HS_API hs_status hs_l21_grad(hs_plan_t plan, const void* A, const void* w_rows, void* out, void* stream);
 
 /*
+ * hs_l21_grad_scaled - hs_l21_grad times a factor that lives on the device (one
+ * real of the plan's precision): the backward pass of the l2,1 norm for an
+ * incoming gradient `scale`, without a second pass over the coefficients.
+ */
+HS_API hs_status hs_l21_grad_scaled(hs_plan_t plan, const void* A, const void* w_rows, const void* scale, void* out,
+                                    void* stream);
+
+/*
  * hs_prox_nuclear - singular value soft threshold of the N x L matrix whose
  * column l is channel l (Eq. "prox-L*"), through the L x L Gram matrix
  * Z^T Z (FP64 accumulation) and its FP64 Jacobi eigendecomposition:

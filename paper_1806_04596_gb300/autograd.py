@@ -94,8 +94,9 @@ class _L21Norm(torch.autograd.Function):
     @staticmethod
     def backward(ctx, g):
         (A,) = ctx.saved_tensors
-        d = ctx.plan.l21_grad(_c(A), ctx.w_rows)
-        return d * g, None, None
+        if torch.is_grad_enabled():   # create_graph: keep the product with g differentiable
+            return ctx.plan.l21_grad(_c(A), ctx.w_rows) * g, None, None
+        return ctx.plan.l21_grad(_c(A), ctx.w_rows, scale=_c(g)), None, None
 
 
 class _Gram(torch.autograd.Function):

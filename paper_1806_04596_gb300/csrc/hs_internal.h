@@ -269,8 +269,9 @@ hs_status dwt_analysis(Plan* p, const void* X, void* A, cudaStream_t s);
 hs_status dwt_synthesis(Plan* p, const void* A, void* X, cudaStream_t s);
 
 // Proximal operators and PD pieces (hs_prox.cu)
+// gscale: device real multiplying every output, or null.
 hs_status l21_apply(Plan* p, const void* A, const void* Wadd, const void* w_rows, double thr,
-                    int dual, void* out, cudaStream_t s);
+                    int dual, void* out, cudaStream_t s, const void* gscale = nullptr);
 hs_status l21_norm(Plan* p, const void* A, const void* w_rows, double* out_dev, cudaStream_t s);
 hs_status nuclear_svals(Plan* p, const void* X, double* sv_out, cudaStream_t s);
 hs_status reweight_rows(Plan* p, const void* A, double gamma, void* w_out, cudaStream_t s);

@@ -37,10 +37,10 @@ __global__ void k_reduce_rows(const double* __restrict__ part, int nb, double* _
 // over the L channels (stride N), the row norm, and the scaled row. For
 // L <= LMAX the row is held in registers (each input read once); LMAX = 0 is
 // the general form that reads the row twice.
-template <typename R, int LMAX>
+template <typename R, int LMAX, bool SCALED>
 __global__ void __launch_bounds__(256) k_l21(const R* __restrict__ A, const R* __restrict__ W,
                                              const R* __restrict__ w_rows, R thr, int dual,
-                                             R* __restrict__ out, int L, int64_t N) {
+                                             const R* __restrict__ gscale, R* __restrict__ out, int L, int64_t N) {
     const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (t >= (int64_t)NB * N) return;
     const int b = (int)(t / N);
@@ -72,15 +72,16 @@ __global__ void __launch_bounds__(256) k_l21(const R* __restrict__ A, const R* _
     if (dual == 2) f = (nrm > (R)0) ? lam / nrm : (R)0;   // direction: gradient of lam ||q||
     else if (dual) f = (nrm > lam) ? lam / nrm : (R)1;
     else f = (nrm > lam) ? (nrm - lam) / nrm : (R)0;
+    const R gs = SCALED ? *gscale : (R)1;
     if (LMAX > 0) {
 #pragma unroll
         for (int l = 0; l < LMAX; ++l)
-            if (l < L) out[base + (int64_t)l * N] = q[l] * f;
+            if (l < L) out[base + (int64_t)l * N] = SCALED ? q[l] * f * gs : q[l] * f;
     } else {
         for (int l = 0; l < L; ++l) {
             R v = A[base + (int64_t)l * N];
             if (W) v += W[base + (int64_t)l * N];
-            out[base + (int64_t)l * N] = v * f;
+            out[base + (int64_t)l * N] = SCALED ? v * f * gs : v * f;
         }
     }
 }
@@ -92,10 +93,13 @@ __global__ void __launch_bounds__(256) k_l21(const R* __restrict__ A, const R* _
 // same order by every warp. With at most 16 channels of a pair per thread,
 // many more loads are in flight per SM than with a whole row per thread (the
 // kernel streams A and W once and writes the dual once).
-template <int LW>
+// SCALED: *gscale (device) multiplies every output (the incoming gradient of the
+// l2,1 term); a pass of its own over the rows cost 173 us at 512 x 512, L = 32.
+template <int LW, bool SCALED>
 __global__ void __launch_bounds__(128) k_l21_split(const float* __restrict__ A, const float* __restrict__ W,
                                                    const float* __restrict__ w_rows, float thr, int dual,
-                                                   float* __restrict__ out, int L, int64_t N) {
+                                                   const float* __restrict__ gscale, float* __restrict__ out, int L,
+                                                   int64_t N) {
     __shared__ float2 part[4][32];
     const int64_t Nh = N >> 1;
     const int64_t nq = (Nh + 31) >> 5;   // CTAs per basis
@@ -141,12 +145,92 @@ __global__ void __launch_bounds__(128) k_l21_split(const float* __restrict__ A, 
         f0 = (n0 > lam0) ? (n0 - lam0) / n0 : 0.f;
         f1 = (n1 > lam1) ? (n1 - lam1) / n1 : 0.f;
     }
+    const float gs = SCALED ? *gscale : 1.f;
 #pragma unroll
     for (int c = 0; c < LW; ++c) {
         const int l = wv + 4 * c;
-        if (l < L)
-            *reinterpret_cast<float2*>(out + base + (int64_t)l * N) = make_float2(q[c].x * f0, q[c].y * f1);
+        if (l < L) {
+            float2 o = make_float2(q[c].x * f0, q[c].y * f1);
+            if (SCALED) o = make_float2(o.x * gs, o.y * gs);
+            *reinterpret_cast<float2*>(out + base + (int64_t)l * N) = o;
+        }
     }
+}
+
+// (hi, lo) += x exactly up to the rounding of lo (Knuth's two-sum).
+__device__ __forceinline__ void pair_add(float& hi, float& lo, float x) {
+    const float s = __fadd_rn(hi, x), t = __fsub_rn(s, hi);
+    lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(s, t)), __fsub_rn(x, t)));
+    hi = s;
+}
+
+// l2,1 norm of an FP32 cube in pairs of FP32 values. FP64 runs at 1/64 of the FP32
+// rate, and one conversion and one FP64 multiply-add per coefficient bounded the plain
+// form below (386 us at 512 x 512, L = 32, now 62: 302 MB that stream in 45). Here a square is
+// a pair p + e, exact (e from the fused multiply-add), and pairs are added with the
+// error-free two-sum; the root is an FP32 value r rounded from a Newton step plus the
+// correction (s - r^2) / 2r (its own error below 2^-49 of r); rows are added in pairs
+// too, and FP64 only sees one pair per thread. A lane owns two neighbouring rows at a
+// time and 16 of their channels are in flight (the 4-warp split of k_l21_split, with its
+// two barriers per tile, took 148 us here). Rows whose squares leave the range in which
+// p + e is exact (or are not finite) are summed again in FP64.
+__global__ void __launch_bounds__(256) k_l21_norm_pairs(const float* __restrict__ A,
+                                                        const float* __restrict__ w_rows, int L, int64_t N,
+                                                        double* __restrict__ part) {
+    __shared__ double red[32];
+    const int64_t Nh = N >> 1;
+    double acc = 0.0;               // rows outside the range
+    float ahi = 0.f, alo = 0.f;     // the others
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < NB * Nh;
+         i += (int64_t)gridDim.x * blockDim.x) {
+        const int b = (int)(i / Nh);
+        const int64_t pix = 2 * (i - (int64_t)b * Nh);
+        const float* row = A + (int64_t)b * L * N + pix;
+        float hi[2] = {0.f, 0.f}, lo[2] = {0.f, 0.f}, mx[2] = {0.f, 0.f};
+        for (int l0 = 0; l0 < L; l0 += 16) {
+            float2 v[16];
+#pragma unroll
+            for (int c = 0; c < 16; ++c)
+                v[c] = l0 + c < L ? *reinterpret_cast<const float2*>(row + (int64_t)(l0 + c) * N)
+                                  : make_float2(0.f, 0.f);
+#pragma unroll
+            for (int c = 0; c < 16; ++c) {
+                const float q[2] = {v[c].x, v[c].y};
+#pragma unroll
+                for (int k = 0; k < 2; ++k) {
+                    const float p = __fmul_rn(q[k], q[k]);
+                    lo[k] = __fadd_rn(lo[k], __fmaf_rn(q[k], q[k], -p));
+                    pair_add(hi[k], lo[k], p);
+                    mx[k] = fmaxf(mx[k], fabsf(q[k]));
+                }
+            }
+        }
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            const float s = hi[k];
+            const float wr = w_rows ? w_rows[(int64_t)b * N + pix + k] : 1.f;
+            if (s >= 0x1p-85f && s <= 0x1p126f && fabsf(wr) <= 0x1p60f && (fabsf(wr) >= 0x1p-40f || wr == 0.f)) {
+                const float y = rsqrtf(s), h = 0.5f * y;
+                float r = s * y;
+                r = fmaf(h, fmaf(-r, r, s), r);
+                const float c = h * (__fmaf_rn(-r, r, s) + lo[k]);   // root = r + c
+                const float p = __fmul_rn(r, wr);
+                alo = __fadd_rn(alo, fmaf(c, wr, __fmaf_rn(r, wr, -p)));
+                pair_add(ahi, alo, p);
+            } else if (mx[k] != 0.f || !(s == 0.f)) {
+                double d = 0.0;
+                for (int l = 0; l < L; ++l) {
+                    const double q = (double)row[(int64_t)l * N + k];
+                    d += q * q;
+                }
+                acc += sqrt(d) * (double)wr;
+            } else {
+                acc += 0.0 * (double)wr;   // a zero row (NaN for a non-finite weight)
+            }
+        }
+    }
+    acc = block_sum(acc + ((double)ahi + (double)alo), red);
+    if (threadIdx.x == 0) part[blockIdx.x] = acc;
 }
 
 template <typename R>
@@ -171,24 +255,33 @@ __global__ void k_l21_norm(const R* __restrict__ A, const R* __restrict__ w_rows
 }
 
 hs_status l21_apply(Plan* p, const void* A, const void* Wadd, const void* w_rows, double thr,
-                    int dual, void* out, cudaStream_t s) {
+                    int dual, void* out, cudaStream_t s, const void* gscale) {
     const int64_t N = p->N();
     const unsigned g = nblk((int64_t)NB * N, 256);
     const int L = p->g.L;
-#define HS_L21(R, LM)                                                                                    \
-    k_l21<R, LM><<<g, 256, 0, s>>>((const R*)A, (const R*)Wadd, (const R*)w_rows, (R)thr, dual, (R*)out, L, \
-                                   N)
+#define HS_L21S(R, LM, SC)                                                                          \
+    k_l21<R, LM, SC><<<g, 256, 0, s>>>((const R*)A, (const R*)Wadd, (const R*)w_rows, (R)thr, dual, \
+                                       (const R*)gscale, (R*)out, L, N)
+#define HS_L21(R, LM)                         \
+    do {                                      \
+        if (gscale) HS_L21S(R, LM, true);     \
+        else HS_L21S(R, LM, false);           \
+    } while (0)
+#define HS_L21P(LW, SC)                                                                                \
+    k_l21_split<LW, SC><<<g2, 128, 0, s>>>((const float*)A, (const float*)Wadd, (const float*)w_rows, \
+                                           (float)thr, dual, (const float*)gscale, (float*)out, L, N)
     auto al8 = [](const void* q) { return ((uintptr_t)q % 8) == 0; };
     const bool pairs = (N % 2) == 0 && al8(A) && al8(Wadd) && al8(w_rows) && al8(out);
     if (p->prec == HS_F32 && pairs && L <= 64) {
         const int64_t nq = (N / 2 + 31) / 32;
         const unsigned g2 = (unsigned)(NB * nq);
-        if (L <= 16)
-            k_l21_split<4><<<g2, 128, 0, s>>>((const float*)A, (const float*)Wadd, (const float*)w_rows,
-                                              (float)thr, dual, (float*)out, L, N);
-        else
-            k_l21_split<16><<<g2, 128, 0, s>>>((const float*)A, (const float*)Wadd, (const float*)w_rows,
-                                               (float)thr, dual, (float*)out, L, N);
+        if (L <= 16) {
+            if (gscale) HS_L21P(4, true);
+            else HS_L21P(4, false);
+        } else {
+            if (gscale) HS_L21P(16, true);
+            else HS_L21P(16, false);
+        }
     } else if (p->prec == HS_F32) {
         if (L <= 16) HS_L21(float, 16);
         else if (L <= 64) HS_L21(float, 64);
@@ -198,6 +291,8 @@ hs_status l21_apply(Plan* p, const void* A, const void* Wadd, const void* w_rows
         else if (L <= 64) HS_L21(double, 64);
         else HS_L21(double, 0);
     }
+#undef HS_L21S
+#undef HS_L21P
 #undef HS_L21
     HS_CHECK_LAUNCH();
     return HS_OK;
@@ -234,8 +329,11 @@ hs_status l1_apply(Plan* p, const void* A, const void* Wadd, const void* w, doub
 
 hs_status l21_norm(Plan* p, const void* A, const void* w_rows, double* out_dev, cudaStream_t s) {
     const int64_t N = p->N();
-    const int nb = 512;
-    if (p->prec == HS_F32)
+    int nb = 512;
+    if (p->prec == HS_F32 && N % 2 == 0 && (uintptr_t)A % 8 == 0) {
+        nb = (int)std::min<int64_t>(nblk(NB * (N / 2), 256), 152 * 6);
+        k_l21_norm_pairs<<<nb, 256, 0, s>>>((const float*)A, (const float*)w_rows, p->g.L, N, p->part);
+    } else if (p->prec == HS_F32)
         k_l21_norm<float><<<nb, 256, 0, s>>>((const float*)A, (const float*)w_rows, p->g.L, N, p->part);
     else
         k_l21_norm<double><<<nb, 256, 0, s>>>((const double*)A, (const double*)w_rows, p->g.L, N,
@@ -474,6 +572,75 @@ __global__ void __launch_bounds__(256) k_gram(const R* __restrict__ X, const R* 
         }
 }
 
+// FP64 form: only the upper triangle's 4 x 4 blocks, P = nb (nb + 1) / 2 of nb = ceil(L / 4)
+// block rows, and the 256 threads split the pixels of a tile 256 / P ways (FP64 issues
+// at 1/64 of the FP32 rate, so every multiply-add of a padded or mirrored block costs:
+// 128 x 128, L = 6 took 171 us with the 16 x 16 block grid above, now 13). Each thread sums its
+// share of a tile in FP64 and adds it to its total; the shares meet in shared memory.
+__global__ void __launch_bounds__(256) k_gram_f64(const double* __restrict__ X, const double* __restrict__ Xa, int L,
+                                                  int64_t N, double* __restrict__ part) {
+    __shared__ __align__(16) double zs[GRAM_PIX * GRAM_LDZ];   // pixel-major tile, then the shares
+    const int tid = threadIdx.x;
+    const int nb = (L + 3) >> 2, P = nb * (nb + 1) / 2, S = 256 / P;
+    const int pr = tid % P, sl = tid / P;   // block and pixel share of this thread (sl < S)
+    int bi = 0, rem = pr;
+    while (rem >= nb - bi) rem -= nb - bi++;
+    const int bj = bi + rem;
+    double tot[16];
+#pragma unroll
+    for (int q = 0; q < 16; ++q) tot[q] = 0.0;
+    const int LP = 4 * nb;                    // channels staged (zeros above L)
+    const int64_t ntile = N / GRAM_PIX;
+    const int px0 = tid & (GRAM_PIX - 1), l0 = tid >> 6;
+    for (int64_t tile = blockIdx.x; tile < ntile; tile += gridDim.x) {
+        const int64_t n = tile * GRAM_PIX + px0;
+        __syncthreads();
+        for (int l = l0; l < LP; l += 4) {
+            double z = 0.0;
+            if (l < L) {
+                z = X[(int64_t)l * N + n];
+                if (Xa) z += Xa[(int64_t)l * N + n];
+            }
+            zs[px0 * GRAM_LDZ + l] = z;
+        }
+        __syncthreads();
+        if (sl < S) {
+            double acc[16];
+#pragma unroll
+            for (int q = 0; q < 16; ++q) acc[q] = 0.0;
+            for (int px = sl; px < GRAM_PIX; px += S) {
+                double a[4], b[4];
+                ld4(&zs[px * GRAM_LDZ + 4 * bi], a);
+                ld4(&zs[px * GRAM_LDZ + 4 * bj], b);
+#pragma unroll
+                for (int t = 0; t < 4; ++t)
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) acc[4 * t + u] = fma(a[t], b[u], acc[4 * t + u]);
+            }
+#pragma unroll
+            for (int q = 0; q < 16; ++q) tot[q] += acc[q];
+        }
+    }
+    __syncthreads();
+    if (sl < S)
+#pragma unroll
+        for (int q = 0; q < 16; ++q) zs[(q * S + sl) * P + pr] = tot[q];
+    __syncthreads();
+    for (int o = tid; o < 16 * P; o += 256) {   // one entry of one block per thread
+        const int q = o / P, pb = o - q * P;
+        int oi = 0, om = pb;
+        while (om >= nb - oi) om -= nb - oi++;
+        const int i = 4 * oi + (q >> 2), j = 4 * (oi + om) + (q & 3);
+        if (i <= j && j < L) {
+            double v = 0.0;
+            for (int k = 0; k < S; ++k) v += zs[(q * S + k) * P + pb];
+            const int e = i * L - i * (i - 1) / 2 + (j - i);
+            part[(int64_t)e * gridDim.x + blockIdx.x] = v;
+        }
+    }
+}
+static_assert(16 * 256 <= GRAM_PIX * GRAM_LDZ, "the shares fit the tile");
+
 // Sum the per-CTA partials (fixed order) and expand to the full symmetric matrix.
 __global__ void k_gram_reduce(const double* __restrict__ part, int nb, int L, double* __restrict__ S) {
     __shared__ double red[32];
@@ -684,7 +851,7 @@ hs_status gram_matrix(Plan* p, const void* X, const void* Xadd, cudaStream_t s) 
     } else if (p->prec == HS_F32) {
         k_gram<float><<<GRAM_CTAS, 256, 0, s>>>((const float*)X, (const float*)Xadd, L, N, p->part);
     } else {
-        k_gram<double><<<GRAM_CTAS, 256, 0, s>>>((const double*)X, (const double*)Xadd, L, N, p->part);
+        k_gram_f64<<<GRAM_CTAS, 256, 0, s>>>((const double*)X, (const double*)Xadd, L, N, p->part);
     }
     HS_CHECK_LAUNCH();
     k_gram_reduce<<<P, 128, 0, s>>>(p->part, nb, L, p->gram);
