@@ -512,6 +512,387 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 4 : 1)
     tile_store<R>(cl, acc, X + l * N + t0, A + l * N + t0, nx, qy, qx, s);
 }
 
+// ---- FP32 levels of whole 32 x 32 coefficient tiles (64 x 64 samples per CTA)
+// The 16 x 16 tiles above are issue bound, and a third of their instructions are filter
+// taps: the rest is staging (46^2 samples for 32^2), addresses, short loops. With four
+// times the tile a column thread makes 4 output rows from F + 6 loads (2 from F + 2), the
+// halo shrinks (78^2 for 64^2) and stores are whole 128-byte rows. The taps are added in
+// the same order, so every coefficient is the same bits. us per
+// direction, before -> after: 1024 x 1024, L = 16 412 -> 277 and 528 -> 364; 512 x 512,
+// L = 32 207 -> 148 and 273 -> 205; 256 x 256, L = 60 97 -> 79 and 128 -> 115.
+constexpr int BQ = 32;                    // coefficients per subband and axis in one tile
+constexpr int BIN = 2 * BQ + MAXF - 2;    // analysis input region side (78)
+constexpr int BSI = BIN + 4;              // its row stride (82 = 18 mod 32: pair loads of 4 rows x 4 groups hit distinct banks)
+constexpr int BSR = 80;                   // row-filtered tile stride: lowpass at 0, highpass at 32
+constexpr int BFWD_SMEM = BIN * BSI + BIN * BSR;   // floats
+constexpr int BC = BQ + MAXF / 2 - 1;     // synthesis coefficient region side (39)
+constexpr int BSC = 44;                   // row stride of the staged coefficients (16-byte chunks)
+constexpr int BSH = 40;                   // columns of a column-filtered half
+constexpr int BSL = 2 * BSH + 1;          // column-filtered tile stride
+constexpr int BINV_SMEM = 4 * BC * BSC + 2 * BQ * BSL;   // floats
+static_assert(2 * BQ * (2 * BQ + 1) <= 2 * BQ * BSL, "output transpose fits the column tile");
+
+template <bool P2>
+__device__ __forceinline__ void big_stage(float* in, const float* __restrict__ base, int64_t stride, int ysz, int xsz,
+                                          int y0, int x0, int ry, int rx, bool pairs) {
+    const int lane = threadIdx.x & 31, wy = threadIdx.x >> 5;
+    for (int r = wy; r < ry; r += 8) {
+        const float* row = base + (int64_t)wrapp<P2>(y0 + r, ysz) * stride;
+        float* d = in + r * BSI;
+        if (pairs)
+            for (int c = 2 * lane; c < rx; c += 64) cp_async8(d + c, row + wrapp<P2>(x0 + c, xsz));
+        else
+            for (int c = lane; c < rx; c += 32) cp_async(d + c, row + wrapp<P2>(x0 + c, xsz));
+    }
+    cp_async_commit();
+}
+
+// Analysis along x: a task is one row and one half of its columns, 4 lanes to a task,
+// each making 4 lowpass and 4 highpass outputs.
+template <int D> __device__ __forceinline__ void big_rows(const float* __restrict__ in, float* __restrict__ ro) {
+    constexpr int F = 2 * (D + 1), NV = F + 6, RY = 2 * BQ + F - 2;
+    for (int t = threadIdx.x >> 2; t < 2 * RY; t += 64) {
+        const int h = t >= RY, r = t - h * RY, g = 4 * h + (threadIdx.x & 3);
+        float v[NV];
+        const float* p = in + r * BSI + 8 * g;
+#pragma unroll
+        for (int k = 0; k < NV / 2; ++k) {
+            const float2 q = ld2(p + 2 * k);
+            v[2 * k] = q.x;
+            v[2 * k + 1] = q.y;
+        }
+        float lo[4], hi[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            float a = 0, b = 0;
+#pragma unroll
+            for (int j = 0; j < F; ++j) {
+                a = fma(filt<float>(D, 0, j), v[2 * u + j], a);
+                b = fma(filt<float>(D, 1, j), v[2 * u + j], b);
+            }
+            lo[u] = a;
+            hi[u] = b;
+        }
+        st4(ro + r * BSR + 4 * g, lo[0], lo[1], lo[2], lo[3]);
+        st4(ro + r * BSR + BQ + 4 * g, hi[0], hi[1], hi[2], hi[3]);
+    }
+}
+
+// Analysis along y and the subband stores: a thread makes output rows 4g .. 4g + 3 of tile
+// column col (0-31: x-lowpass, 32-63: x-highpass) for two g.
+template <int D>
+__device__ __forceinline__ void big_cols(const float* __restrict__ ro, float sc, float* __restrict__ Ad,
+                                         float* __restrict__ LLo, int64_t lls, int nx, int hy, int hx, int k0y,
+                                         int k0x) {
+    constexpr int F = 2 * (D + 1), NV = F + 6;
+    const int col = threadIdx.x & 63, c = col & 31;
+    const bool xhi = col >= 32;
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+        const int g = (threadIdx.x >> 6) + 4 * i;
+        float v[NV];
+#pragma unroll
+        for (int k = 0; k < NV; ++k) v[k] = ro[(8 * g + k) * BSR + col];
+        const int oy = k0y + 4 * g;
+        float* lo = xhi ? Ad + (int64_t)oy * nx + hx + k0x + c : LLo + (int64_t)oy * lls + k0x + c;
+        float* hi = Ad + (int64_t)(hy + oy) * nx + (xhi ? hx : 0) + k0x + c;
+        const int64_t ls = xhi ? nx : lls;
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            float a = 0, b = 0;
+#pragma unroll
+            for (int j = 0; j < F; ++j) {
+                a = fma(filt<float>(D, 0, j), v[2 * u + j], a);
+                b = fma(filt<float>(D, 1, j), v[2 * u + j], b);
+            }
+            lo[u * ls] = sc * a;
+            hi[(int64_t)u * nx] = sc * b;
+        }
+    }
+}
+
+struct BigFwd {
+    const float* in;
+    float* ro;
+    float* A;
+    float* ll_out;
+    int64_t N;
+    int L, l, nx, hy, hx, k0y, k0x, last;
+    float sc;
+};
+template <int D> __device__ __forceinline__ void big_fwd_all(const BigFwd& c) {
+    if constexpr (D < NW) {
+        big_rows<D>(c.in, c.ro);
+        __syncthreads();
+        float* Ad = c.A + ((int64_t)(1 + D) * c.L + c.l) * c.N;
+        float* LLo = c.last ? Ad : c.ll_out + ((int64_t)D * c.L + c.l) * (int64_t)c.hy * c.hx;
+        big_cols<D>(c.ro, c.sc, Ad, LLo, c.last ? c.nx : c.hx, c.nx, c.hy, c.hx, c.k0y, c.k0x);
+        __syncthreads();
+        big_fwd_all<D + 1>(c);
+    }
+}
+
+// k_psi_fwd_l0 on 32 x 32 tiles.
+template <bool P2>
+__global__ void __launch_bounds__(256, 4) k_psi_fwd_l0_big(const float* __restrict__ X, float* __restrict__ A,
+                                                          float* __restrict__ ll_out, int L, int ny, int nx, int last,
+                                                          float sc, int pairs) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    float* in = reinterpret_cast<float*>(smem_raw);
+    const int lane = threadIdx.x & 31, wy = threadIdx.x >> 5;
+    const int l = blockIdx.y;
+    const int hy = ny >> 1, hx = nx >> 1, ntx = hx / BQ;
+    const int ty = blockIdx.x / ntx, tx = blockIdx.x - ty * ntx;
+    const int k0y = ty * BQ, k0x = tx * BQ;
+    const int64_t N = (int64_t)ny * nx;
+    big_stage<P2>(in, X + l * N, nx, ny, nx, 2 * k0y, 2 * k0x, BIN, BIN, pairs != 0);
+    cp_async_wait<0>();
+    __syncthreads();
+    float* A0 = A + l * N + (int64_t)(2 * k0y) * nx + 2 * k0x;
+    for (int r = wy; r < 2 * BQ; r += 8)
+        for (int c = lane; c < 2 * BQ; c += 32) A0[(int64_t)r * nx + c] = sc * in[r * BSI + c];
+    BigFwd c{in, in + BIN * BSI, A, ll_out, N, L, l, nx, hy, hx, k0y, k0x, last, sc};
+    big_fwd_all<0>(c);
+}
+
+// k_dwt_fwd_level on 32 x 32 tiles.
+template <bool P2>
+__global__ void __launch_bounds__(256, 4) k_dwt_fwd_level_big(const float* __restrict__ src, float* __restrict__ A,
+                                                             float* __restrict__ ll_out, int L, int ny, int nx, int my,
+                                                             int mx, int last) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    float* in = reinterpret_cast<float*>(smem_raw);
+    float* ro = in + BIN * BSI;
+    const int d = blockIdx.y / L, l = blockIdx.y - d * L;
+    const int hy = my >> 1, hx = mx >> 1, ntx = hx / BQ;
+    const int ty = blockIdx.x / ntx, tx = blockIdx.x - ty * ntx;
+    const int k0y = ty * BQ, k0x = tx * BQ;
+    const int64_t N = (int64_t)ny * nx;
+    const float* base = src + ((int64_t)d * L + l) * (int64_t)my * mx;
+    float* Ad = A + ((int64_t)(1 + d) * L + l) * N;
+    float* LLo = last ? Ad : ll_out + ((int64_t)d * L + l) * (int64_t)hy * hx;
+    const int64_t lls = last ? nx : hx;
+#define HS_FWD(DD)                                                                                          \
+    {                                                                                                       \
+        constexpr int F = 2 * (DD + 1);                                                                     \
+        big_stage<P2>(in, base, mx, my, mx, 2 * k0y, 2 * k0x, 2 * BQ + F - 2, 2 * BQ + F - 2, true);        \
+        cp_async_wait<0>();                                                                                 \
+        __syncthreads();                                                                                    \
+        big_rows<DD>(in, ro);                                                                               \
+        __syncthreads();                                                                                    \
+        big_cols<DD>(ro, 1.f, Ad, LLo, lls, nx, hy, hx, k0y, k0x);                                          \
+    }
+    HS_DWT_DISPATCH(d, HS_FWD)
+#undef HS_FWD
+}
+
+// Stages the four subband regions of one (d, l) tile (inv_stage on 32 x 32 tiles).
+template <int D, bool P2>
+__device__ __forceinline__ void big_inv_stage(float* cf, const float* __restrict__ Ad, const float* __restrict__ ll,
+                                              int64_t lls, int nx, int hy, int hx, int ky0, int kx0, bool chunks) {
+    constexpr int CO = inv_co<float, D>(), CN = BQ + D, NCH = (CN + CO + 3) / 4;
+    const int lane = threadIdx.x & 31, wy = threadIdx.x >> 5;
+    if (chunks) {   // 16 lanes per row
+        const int cc = lane & 15, rr = lane >> 4;
+        const int gx = wrapp<P2>(kx0 - CO + 4 * cc, hx);
+        if (cc < NCH)
+#pragma unroll
+            for (int s = 0; s < 4; ++s)
+                for (int yy = 2 * wy + rr; yy < CN; yy += 16) {
+                    const int gy = wrapp<P2>(ky0 + yy, hy);
+                    const float* src = (s == 0) ? ll + (int64_t)gy * lls + gx
+                                                : Ad + (int64_t)((s >> 1) * hy + gy) * nx + (s & 1) * hx + gx;
+                    cp_async16(cf + (s * BC + yy) * BSC + 4 * cc, src);
+                }
+    } else {
+#pragma unroll
+        for (int s = 0; s < 4; ++s)
+            for (int yy = wy; yy < CN; yy += 8) {
+                const int gy = wrapp<P2>(ky0 + yy, hy);
+                for (int c = lane; c < CN; c += 32) {
+                    const int gx = wrapp<P2>(kx0 + c, hx);
+                    const float* src = (s == 0) ? ll + (int64_t)gy * lls + gx
+                                                : Ad + (int64_t)((s >> 1) * hy + gy) * nx + (s & 1) * hx + gx;
+                    cp_async(cf + (s * BC + yy) * BSC + CO + c, src);
+                }
+            }
+    }
+    cp_async_commit();
+}
+
+// Synthesis along y (inv_cols): a task is one column of one half and 4 coefficient rows.
+template <int D> __device__ __forceinline__ void big_inv_cols(const float* __restrict__ cf, float* __restrict__ cl) {
+    constexpr int H = D + 1, NV = H + 3, CN = BQ + D;
+    for (int t = threadIdx.x; t < CN * 2 * (BQ / 4); t += 256) {
+        const int q = t / CN, x = t - q * CN, b = q & 1, m0 = 4 * (q >> 1);
+        float a[NV], e[NV];
+#pragma unroll
+        for (int k = 0; k < NV; ++k) {
+            a[k] = cf[(b * BC + m0 + k) * BSC + inv_co<float, D>() + x];
+            e[k] = cf[((2 + b) * BC + m0 + k) * BSC + inv_co<float, D>() + x];
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            float v0 = 0, v1 = 0;
+#pragma unroll
+            for (int k = 0; k < H; ++k) {
+                const int i = u - k + H - 1;
+                v0 = fma(filt<float>(D, 0, 2 * k), a[i], v0);
+                v0 = fma(filt<float>(D, 1, 2 * k), e[i], v0);
+                v1 = fma(filt<float>(D, 0, 2 * k + 1), a[i], v1);
+                v1 = fma(filt<float>(D, 1, 2 * k + 1), e[i], v1);
+            }
+            cl[(2 * (m0 + u)) * BSL + b * BSH + x] = v0;
+            cl[(2 * (m0 + u) + 1) * BSL + b * BSH + x] = v1;
+        }
+    }
+}
+
+// Synthesis along x (inv_rows): thread (i, g) adds output columns 8n .. 8n + 7 of tile row i
+// into acc[8 it ..], n = g + 4 it.
+template <int D> __device__ __forceinline__ void big_inv_rows(const float* __restrict__ cl, float* acc) {
+    constexpr int H = D + 1, NV = H + 3;
+    const int i = threadIdx.x & 63;
+#pragma unroll
+    for (int it = 0; it < 2; ++it) {
+        const int n0 = 4 * ((threadIdx.x >> 6) + 4 * it);
+        float a[NV], e[NV];
+#pragma unroll
+        for (int k = 0; k < NV; ++k) {
+            a[k] = cl[i * BSL + n0 + k];
+            e[k] = cl[i * BSL + BSH + n0 + k];
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            float v0 = 0, v1 = 0;
+#pragma unroll
+            for (int k = 0; k < H; ++k) {
+                const int t = u - k + H - 1;
+                v0 = fma(filt<float>(D, 0, 2 * k), a[t], v0);
+                v0 = fma(filt<float>(D, 1, 2 * k), e[t], v0);
+                v1 = fma(filt<float>(D, 0, 2 * k + 1), a[t], v1);
+                v1 = fma(filt<float>(D, 1, 2 * k + 1), e[t], v1);
+            }
+            acc[8 * it + 2 * u] += v0;
+            acc[8 * it + 2 * u + 1] += v1;
+        }
+    }
+}
+
+// tile_store for the 64 x 64 tile held as big_inv_rows leaves it.
+__device__ __forceinline__ void big_tile_store(float* T, const float* acc, float* __restrict__ out,
+                                               const float* __restrict__ add, int64_t stride, float s) {
+    constexpr int ST = 2 * BQ + 1;
+    const int i = threadIdx.x & 63;
+#pragma unroll
+    for (int it = 0; it < 2; ++it)
+#pragma unroll
+        for (int u = 0; u < 8; ++u) T[i * ST + 8 * ((threadIdx.x >> 6) + 4 * it) + u] = acc[8 * it + u];
+    __syncthreads();
+    const int lane = threadIdx.x & 31, wy = threadIdx.x >> 5;
+    for (int r = wy; r < 2 * BQ; r += 8)
+        for (int c = lane; c < 2 * BQ; c += 32) {
+            const int64_t o = (int64_t)r * stride + c;
+            float v = T[r * ST + c];
+            if (add) v += add[o];
+            out[o] = s * v;
+        }
+}
+
+// k_dwt_inv_level on 32 x 32 tiles.
+template <bool P2>
+__global__ void __launch_bounds__(256, 4)
+    k_dwt_inv_level_big(const float* __restrict__ A, const float* __restrict__ llbuf, int ll_from_a,
+                        float* __restrict__ out, int L, int ny, int nx, int my, int mx, int chunks) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    float* cf = reinterpret_cast<float*>(smem_raw);
+    float* cl = cf + 4 * BC * BSC;
+    const int d = blockIdx.y / L, l = blockIdx.y - d * L;
+    const int hy = my >> 1, hx = mx >> 1, ntx = hx / BQ;
+    const int ty = blockIdx.x / ntx, tx = blockIdx.x - ty * ntx;
+    const int64_t N = (int64_t)ny * nx;
+    const float* Ad = A + ((int64_t)(1 + d) * L + l) * N;
+    const float* ll = ll_from_a ? Ad : llbuf + ((int64_t)d * L + l) * (int64_t)hy * hx;
+    float acc[16];
+#pragma unroll
+    for (int k = 0; k < 16; ++k) acc[k] = 0.f;
+#define HS_INV(DD)                                                                                     \
+    {                                                                                                  \
+        big_inv_stage<DD, P2>(cf, Ad, ll, ll_from_a ? nx : hx, nx, hy, hx, ty * BQ - DD, tx * BQ - DD, \
+                              chunks != 0);                                                            \
+        cp_async_wait<0>();                                                                            \
+        __syncthreads();                                                                               \
+        big_inv_cols<DD>(cf, cl);                                                                      \
+        __syncthreads();                                                                               \
+        big_inv_rows<DD>(cl, acc);                                                                     \
+    }
+    HS_DWT_DISPATCH(d, HS_INV)
+#undef HS_INV
+    __syncthreads();
+    float* o = out + ((int64_t)d * L + l) * (int64_t)my * mx + (int64_t)(2 * ty * BQ) * mx + 2 * tx * BQ;
+    big_tile_store(cl, acc, o, nullptr, mx, 1.f);
+}
+
+struct BigInv {
+    float* cf;
+    float* cl;
+    const float* A;
+    const float* llbuf;
+    int64_t N;
+    int L, l, nx, hy, hx, ty, tx, ll_from_a, chunks;
+};
+template <int D, bool P2> __device__ __forceinline__ void big_inv_stage_d(const BigInv& c) {
+    const float* Ad = c.A + ((int64_t)(1 + D) * c.L + c.l) * c.N;
+    const float* ll = c.ll_from_a ? Ad : c.llbuf + ((int64_t)D * c.L + c.l) * (int64_t)c.hy * c.hx;
+    big_inv_stage<D, P2>(c.cf, Ad, ll, c.ll_from_a ? c.nx : c.hx, c.nx, c.hy, c.hx, c.ty * BQ - D, c.tx * BQ - D,
+                         c.chunks != 0);
+}
+// The next wavelet's subbands are staged while the current one is filtered along x.
+template <int D, bool P2> __device__ __forceinline__ void big_inv_all(const BigInv& c, float* acc) {
+    if constexpr (D < NW) {
+        cp_async_wait<0>();
+        __syncthreads();
+        big_inv_cols<D>(c.cf, c.cl);
+        __syncthreads();
+        if constexpr (D + 1 < NW) big_inv_stage_d<D + 1, P2>(c);
+        big_inv_rows<D>(c.cl, acc);
+        big_inv_all<D + 1, P2>(c, acc);
+    }
+}
+
+// k_psi_adj_l0 on 32 x 32 tiles.
+template <bool P2>
+__global__ void __launch_bounds__(256, 4)
+    k_psi_adj_l0_big(const float* __restrict__ A, const float* __restrict__ llbuf, int ll_from_a,
+                     float* __restrict__ X, int L, int ny, int nx, float s, int chunks) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    float* cf = reinterpret_cast<float*>(smem_raw);
+    float* cl = cf + 4 * BC * BSC;
+    const int l = blockIdx.y;
+    const int hy = ny >> 1, hx = nx >> 1, ntx = hx / BQ;
+    const int ty = blockIdx.x / ntx, tx = blockIdx.x - ty * ntx;
+    const int64_t N = (int64_t)ny * nx;
+    BigInv c{cf, cl, A, llbuf, N, L, l, nx, hy, hx, ty, tx, ll_from_a, chunks};
+    big_inv_stage_d<0, P2>(c);
+    float acc[16];
+#pragma unroll
+    for (int k = 0; k < 16; ++k) acc[k] = 0.f;
+    big_inv_all<0, P2>(c, acc);
+    __syncthreads();
+    const int64_t t0 = (int64_t)(2 * ty * BQ) * nx + 2 * tx * BQ;
+    big_tile_store(cl, acc, X + l * N + t0, A + l * N + t0, nx, s);
+}
+
+static inline unsigned big_count(int my, int mx) { return (unsigned)(((my >> 1) / BQ) * ((mx >> 1) / BQ)); }
+
+// FP32 levels whose subbands are whole 32 x 32 tiles, `planes` of them to a launch, where
+// that makes two CTAs per SM (128 x 128, L = 6: 24 CTAs, analysis 15.5 -> 19.5 us;
+// 640 x 384, L = 7: 420 CTAs, 58 -> 45).
+template <typename R> static bool big_tiles(int my, int mx, int planes) {
+    return sizeof(R) == 4 && (my >> 1) % BQ == 0 && (mx >> 1) % BQ == 0 &&
+           (int64_t)big_count(my, mx) * planes >= 2 * 152;
+}
+
 // ---- coarse levels of one (wavelet, channel) in shared memory
 // When a level's input block fits in shared memory, one CTA per (wavelet d,
 // channel l) runs that level and every coarser one without leaving the SM: X
@@ -891,6 +1272,14 @@ hs_status dwt_init() {
     HS_TRY(smem_attr(k_dwt_inv_tail<float, false>, TAIL_SMEM_MAX));
     HS_TRY(smem_attr(k_dwt_inv_tail<double, true>, TAIL_SMEM_MAX));
     HS_TRY(smem_attr(k_dwt_inv_tail<double, false>, TAIL_SMEM_MAX));
+    HS_TRY(smem_attr(k_psi_fwd_l0_big<true>, BFWD_SMEM * 4));
+    HS_TRY(smem_attr(k_psi_fwd_l0_big<false>, BFWD_SMEM * 4));
+    HS_TRY(smem_attr(k_dwt_fwd_level_big<true>, BFWD_SMEM * 4));
+    HS_TRY(smem_attr(k_dwt_fwd_level_big<false>, BFWD_SMEM * 4));
+    HS_TRY(smem_attr(k_psi_adj_l0_big<true>, BINV_SMEM * 4));
+    HS_TRY(smem_attr(k_psi_adj_l0_big<false>, BINV_SMEM * 4));
+    HS_TRY(smem_attr(k_dwt_inv_level_big<true>, BINV_SMEM * 4));
+    HS_TRY(smem_attr(k_dwt_inv_level_big<false>, BINV_SMEM * 4));
     HS_TRY(smem_attr(k_psi_fwd_l0<float, true>, FWD_SMEM * 4));
     HS_TRY(smem_attr(k_psi_fwd_l0<double, true>, FWD_SMEM * 8));
     HS_TRY(smem_attr(k_dwt_fwd_level<float, true>, FWD_SMEM * 4));
@@ -921,15 +1310,26 @@ template <typename R, bool P2> static hs_status analysis_t(Plan* p, const R* X, 
     R* buf[2] = {(R*)p->dwt_a, (R*)p->dwt_b};
     const int top = p->levels - 1;
     const int pairs = ((uintptr_t)X % 8) == 0;   // caller's image: 8-byte pairs only when aligned
-    k_psi_fwd_l0<R, P2><<<dim3(ntiles(ny, nx), L), 256, FWD_SMEM * sizeof(R), s>>>(X, A, buf[0], L, ny, nx, top == 0,
-                                                                              (R)(1.0 / 3.0), pairs);
+    if constexpr (sizeof(R) == 4) {
+        if (big_tiles<R>(ny, nx, L))
+            k_psi_fwd_l0_big<P2><<<dim3(big_count(ny, nx), L), 256, BFWD_SMEM * 4, s>>>(
+                X, A, buf[0], L, ny, nx, top == 0, (R)(1.0 / 3.0), pairs);
+    }
+    if (!big_tiles<R>(ny, nx, L))
+        k_psi_fwd_l0<R, P2><<<dim3(ntiles(ny, nx), L), 256, FWD_SMEM * sizeof(R), s>>>(
+            X, A, buf[0], L, ny, nx, top == 0, (R)(1.0 / 3.0), pairs);
     HS_CHECK_LAUNCH();
     const int t = tail_level<R>(p);
     for (int lev = 1; lev <= top && (t == 0 || lev < t); ++lev) {
         const int my = ny >> lev, mx = nx >> lev;
-        dim3 g(ntiles(my, mx), NW * L);
-        k_dwt_fwd_level<R, P2><<<g, 256, FWD_SMEM * sizeof(R), s>>>(buf[(lev - 1) & 1], A, buf[lev & 1], L, ny, nx,
-                                                                my, mx, lev == top);
+        if constexpr (sizeof(R) == 4) {
+            if (big_tiles<R>(my, mx, NW * L))
+                k_dwt_fwd_level_big<P2><<<dim3(big_count(my, mx), NW * L), 256, BFWD_SMEM * 4, s>>>(
+                    buf[(lev - 1) & 1], A, buf[lev & 1], L, ny, nx, my, mx, lev == top);
+        }
+        if (!big_tiles<R>(my, mx, NW * L))
+            k_dwt_fwd_level<R, P2><<<dim3(ntiles(my, mx), NW * L), 256, FWD_SMEM * sizeof(R), s>>>(
+                buf[(lev - 1) & 1], A, buf[lev & 1], L, ny, nx, my, mx, lev == top);
         HS_CHECK_LAUNCH();
     }
     if (t > 0) {
@@ -955,14 +1355,26 @@ template <typename R, bool P2> static hs_status synthesis_t(Plan* p, const R* A,
     }
     for (int lev = t > 0 ? t - 1 : top; lev >= 1; --lev) {
         const int my = ny >> lev, mx = nx >> lev;
-        dim3 g(ntiles(my, mx), NW * L);
-        k_dwt_inv_level<R, P2><<<g, 256, INV_SMEM * sizeof(R), s>>>(A, lev == top ? nullptr : buf[(lev + 1) & 1],
-                                                                lev == top, buf[lev & 1], L, ny, nx, my, mx,
-                                                                chunks);
+        const R* ll = lev == top ? nullptr : buf[(lev + 1) & 1];
+        if constexpr (sizeof(R) == 4) {
+            if (big_tiles<R>(my, mx, NW * L))
+                k_dwt_inv_level_big<P2><<<dim3(big_count(my, mx), NW * L), 256, BINV_SMEM * 4, s>>>(
+                    A, ll, lev == top, buf[lev & 1], L, ny, nx, my, mx, chunks);
+        }
+        if (!big_tiles<R>(my, mx, NW * L))
+            k_dwt_inv_level<R, P2><<<dim3(ntiles(my, mx), NW * L), 256, INV_SMEM * sizeof(R), s>>>(
+                A, ll, lev == top, buf[lev & 1], L, ny, nx, my, mx, chunks);
         HS_CHECK_LAUNCH();
     }
-    k_psi_adj_l0<R, P2><<<dim3(ntiles(ny, nx), L), 256, INV_SMEM * sizeof(R), s>>>(
-        A, top == 0 ? nullptr : buf[1], top == 0, X, L, ny, nx, (R)(1.0 / 3.0), chunks);
+    const R* ll = top == 0 ? nullptr : buf[1];
+    if constexpr (sizeof(R) == 4) {
+        if (big_tiles<R>(ny, nx, L))
+            k_psi_adj_l0_big<P2><<<dim3(big_count(ny, nx), L), 256, BINV_SMEM * 4, s>>>(
+                A, ll, top == 0, X, L, ny, nx, (R)(1.0 / 3.0), chunks);
+    }
+    if (!big_tiles<R>(ny, nx, L))
+        k_psi_adj_l0<R, P2><<<dim3(ntiles(ny, nx), L), 256, INV_SMEM * sizeof(R), s>>>(
+            A, ll, top == 0, X, L, ny, nx, (R)(1.0 / 3.0), chunks);
     HS_CHECK_LAUNCH();
     return HS_OK;
 }
