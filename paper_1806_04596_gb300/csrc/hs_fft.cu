@@ -48,6 +48,7 @@ template <typename R> struct FftArgs {
     int lgG;           // log2 of the lines per CTA
     int nx, ny, Ky, Kc, Kw;
     int vec;           // the image is aligned for pixel-pair accesses
+    const int4* rng;   // cells reached, per channel
 };
 
 template <typename R> __device__ __forceinline__ Cx<R> twiddle(const Cx<R>* tw, int m, int dir) {
@@ -88,7 +89,7 @@ template <typename R, int DIR> __device__ __forceinline__ void dft5(Cx<R>* a) {
 // The image occupies k < N/4 and k >= 3 N/4 (of a line or of its pixel pairs),
 // so operands 2 .. 5 are zero in the forward modes.
 template <typename R, int MODE>
-__device__ __forceinline__ Cx<R> fft_load(const FftArgs<R>& a, int la, int lb, int N, int k, int r) {
+__device__ __forceinline__ Cx<R> fft_load(const FftArgs<R>& a, const int4& rg, int la, int lb, int N, int k, int r) {
     typedef Cx<R> CT;
     if (MODE == ROW_FWD) {   // Z: pad and scale; pixels 2 m + N/2 (mod 2 N) of row lb
         if (r >= 2 && r < 6) return cx<R>(0, 0);
@@ -105,28 +106,30 @@ __device__ __forceinline__ Cx<R> fft_load(const FftArgs<R>& a, int la, int lb, i
         const int iy = r < 2 ? k + (N >> 2) : k - 3 * (N >> 2);
         return ((const CT*)a.in)[((int64_t)la * a.ny + iy) * a.Kc + lb];
     } else if (MODE == COL_INV) {
+        if (!row_reached(rg, k)) return cx<R>(0, 0);
         return ((const CT*)a.in)[((int64_t)la * a.Ky + k) * a.Kw + lb];
     } else {
         // ROW_INV: fold the mirrored columns (C(k), 0 <= k <= N), then the complex input
         // of the real inverse, ((A + B) + i w (A - B)) / 2 with A = C(k), B = conj C(N - k),
         // w = exp(2 pi i k / 2N) (both ends real and counted twice at k = 0)
         const CT* T = (const CT*)a.in + ((int64_t)la * a.ny + lb) * a.Kc + 3;
+        auto at = [&](int q) { return q + 3 < rg.x ? T[q] : cx<R>(0, 0); };   // rg.y is the pitch here
         auto folded = [&](int q) {
-            CT v = T[q];
+            CT v = at(q);
             if (q <= 3) {
-                const CT m = T[-q];
+                const CT m = at(-q);
                 v.x += m.x;
                 v.y -= m.y;
             }
             if (q >= N - 4) {
-                const CT m = T[2 * N - q];
+                const CT m = at(2 * N - q);
                 v.x += m.x;
                 v.y -= m.y;
             }
             return v;
         };
         if (k == 0) {
-            const R p = T[0].x, q = T[N].x;
+            const R p = at(0).x, q = at(N).x;
             return cx<R>(p + q, p - q);
         }
         const CT A = folded(k);
@@ -140,10 +143,11 @@ __device__ __forceinline__ Cx<R> fft_load(const FftArgs<R>& a, int la, int lb, i
 
 // Last-pass stores of element k (known to lie inside the crop in the inverse modes).
 template <typename R, int MODE>
-__device__ __forceinline__ void fft_store(const FftArgs<R>& a, int la, int lb, int N, int k, bool upper, Cx<R> v) {
+__device__ __forceinline__ void fft_store(const FftArgs<R>& a, const int4& rg, int la, int lb, int N, int k, bool upper,
+                                          Cx<R> v) {
     typedef Cx<R> CT;
     if (MODE == COL_FWD) {
-        ((CT*)a.out)[((int64_t)la * a.Ky + k) * a.Kw + lb] = v;
+        if (row_reached(rg, k)) ((CT*)a.out)[((int64_t)la * a.Ky + k) * a.Kw + lb] = v;
     } else if (MODE == COL_INV) {   // keep the ny image rows
         const int iy = upper ? k - 3 * (N >> 2) : k + (N >> 2);
         ((CT*)a.out)[((int64_t)la * a.ny + iy) * a.Kc + lb] = v;
@@ -171,8 +175,8 @@ template <int ODD, int NREP> __host__ __device__ constexpr int fft_elems() {
 // One Stockham pass of radix RAD with sub-transform length 2^lgNs over the
 // CTA's G lines; LG > 0 fixes N = ODD 2^LG at compile time.
 template <typename R, int DIR, int MODE, int RAD, int LG, int ODD, int NREP, int LGG>
-__device__ __forceinline__ void fft_pass(const FftArgs<R>& a, Cx<R>* sm, int lgNs, bool first, bool last, int la,
-                                         int line0) {
+__device__ __forceinline__ void fft_pass(const FftArgs<R>& a, const int4& rg, Cx<R>* sm, int lgNs, bool first,
+                                         bool last, int la, int line0) {
     typedef Cx<R> CT;
     constexpr bool COLS = (MODE == COL_FWD || MODE == COL_INV);
     constexpr int E = fft_elems<ODD, NREP>();
@@ -194,7 +198,7 @@ __device__ __forceinline__ void fft_pass(const FftArgs<R>& a, Cx<R>* sm, int lgN
 #pragma unroll
         for (int r = 0; r < RAD; ++r) {
             const int k = j + r * nb;
-            v[i * RAD + r] = first ? fft_load<R, MODE>(a, la, line0 + g, N, k, r)
+            v[i * RAD + r] = first ? fft_load<R, MODE>(a, rg, la, line0 + g, N, k, r)
                                    : sm[COLS ? ((lpad(k) << LGG) + g) : (g * LD + lpad(k))];
         }
     }
@@ -247,13 +251,13 @@ __device__ __forceinline__ void fft_pass(const FftArgs<R>& a, Cx<R>* sm, int lgN
             if (!to_global) {
                 sm[COLS ? ((lpad(k) << LGG) + g) : (g * LD + lpad(k))] = u[r];
             } else if (MODE == COL_FWD) {
-                fft_store<R, MODE>(a, la, line0 + g, N, k, false, u[r]);
+                fft_store<R, MODE>(a, rg, la, line0 + g, N, k, false, u[r]);
             } else if (RAD == 8 || RAD == 4) {   // k = j + r N / RAD: the kept quarters are whole operands
-                if (r < RAD / 4) fft_store<R, MODE>(a, la, line0 + g, N, k, false, u[r]);
-                else if (r >= RAD - RAD / 4) fft_store<R, MODE>(a, la, line0 + g, N, k, true, u[r]);
+                if (r < RAD / 4) fft_store<R, MODE>(a, rg, la, line0 + g, N, k, false, u[r]);
+                else if (r >= RAD - RAD / 4) fft_store<R, MODE>(a, rg, la, line0 + g, N, k, true, u[r]);
             } else {
-                if (k < (N >> 2)) fft_store<R, MODE>(a, la, line0 + g, N, k, false, u[r]);
-                else if (k >= 3 * (N >> 2)) fft_store<R, MODE>(a, la, line0 + g, N, k, true, u[r]);
+                if (k < (N >> 2)) fft_store<R, MODE>(a, rg, la, line0 + g, N, k, false, u[r]);
+                else if (k >= 3 * (N >> 2)) fft_store<R, MODE>(a, rg, la, line0 + g, N, k, true, u[r]);
             }
         }
     }
@@ -264,13 +268,14 @@ __device__ __forceinline__ void fft_pass(const FftArgs<R>& a, Cx<R>* sm, int lgN
 // X(k) = (Z(k) + conj Z(N - k)) / 2 + exp(-2 pi i k / 2N) (Z(k) - conj Z(N - k)) / 2i for
 // k = 0 .. N, and X(-k) = conj X(k) in the mirrored columns at both ends.
 template <typename R, int ODD, int NREP>
-__device__ __forceinline__ void row_split(const FftArgs<R>& a, const Cx<R>* sm, int N, int la, int line0) {
+__device__ __forceinline__ void row_split(const FftArgs<R>& a, const int4& rg, const Cx<R>* sm, int N, int la, int line0) {
     typedef Cx<R> CT;
     const int tpr = N / fft_elems<ODD, NREP>();   // threads per row
     const int g = threadIdx.x / tpr, t = threadIdx.x - g * tpr;
     const CT* z = sm + g * (N + (N >> 3));
     CT* out = (CT*)a.out + ((int64_t)la * a.ny + line0 + g) * a.Kc;
     for (int c = t; c < N + 8; c += tpr) {
+        if (c >= rg.x) break;
         const int kx = c - 3;
         const bool mir = kx < 0 || kx > N;
         const int k = kx < 0 ? -kx : (kx > N ? 2 * N - kx : kx);
@@ -304,7 +309,10 @@ __global__ void __launch_bounds__(fft_max_threads<R, ODD, NREP>(), fft_min_ctas<
     constexpr bool COLS = (MODE == COL_FWD || MODE == COL_INV);
     const int la = blockIdx.y;
     const int line0 = COLS ? (blockIdx.x << LGG) : (blockIdx.x << a.lgG);
-#define HS_PASS(RAD, NS, FIRST, LAST) fft_pass<R, DIR, MODE, RAD, LG, ODD, NREP, LGG>(a, sm, NS, FIRST, LAST, la, line0)
+    const int4 rg = a.rng[la];
+    if (COLS && !col_reached(rg, line0)) return;   // the whole group (8 columns divide the bounds)
+#define HS_PASS(RAD, NS, FIRST, LAST) \
+    fft_pass<R, DIR, MODE, RAD, LG, ODD, NREP, LGG>(a, rg, sm, NS, FIRST, LAST, la, line0)
     if constexpr (LG > 0) {
         constexpr int N8 = LG / 3, REM = LG % 3;
 #pragma unroll
@@ -321,7 +329,7 @@ __global__ void __launch_bounds__(fft_max_threads<R, ODD, NREP>(), fft_min_ctas<
     if constexpr (ODD == 3) HS_PASS(3, LG > 0 ? LG : a.lg2, false, true);
     if constexpr (ODD == 5) HS_PASS(5, LG > 0 ? LG : a.lg2, false, true);
 #undef HS_PASS
-    if constexpr (MODE == ROW_FWD) row_split<R, ODD, NREP>(a, sm, LG > 0 ? (ODD << LG) : a.N, la, line0);
+    if constexpr (MODE == ROW_FWD) row_split<R, ODD, NREP>(a, rg, sm, LG > 0 ? (ODD << LG) : a.N, la, line0);
 }
 
 // ---------------------------------------------------------------- launches
@@ -339,9 +347,9 @@ static hs_status run_fft(const FftArgs<R>& a, dim3 grid, int threads, size_t sme
     return HS_OK;
 }
 
-// nl channels starting at in / out (a channel range of the plan's buffers).
+// nl channels from l0, starting at in / out (a channel range of the plan's buffers).
 template <typename R, int DIR, int MODE>
-static hs_status launch_fft(Plan* p, const void* in, void* out, int nl, cudaStream_t s) {
+static hs_status launch_fft(Plan* p, const void* in, void* out, int l0, int nl, cudaStream_t s) {
     constexpr bool cols = (MODE == COL_FWD || MODE == COL_INV);
     FftArgs<R> a{};
     a.in = in;
@@ -356,6 +364,7 @@ static hs_status launch_fft(Plan* p, const void* in, void* out, int nl, cudaStre
     a.tw = (const Cx<R>*)(cols ? p->twy : p->twx);
     a.N = cols ? p->g.Ky : p->g.nx;
     const void* img = MODE == ROW_FWD ? in : out;
+    a.rng = p->rng + l0;
     a.vec = ((uintptr_t)img % sizeof(Cx<R>)) == 0;
     int odd = 1;
     for (int r : {3, 5})
@@ -455,10 +464,10 @@ hs_status fft_init() {
 // Opts the kernels of this plan's line lengths into their shared memory, so that
 // no first launch inside a stream capture has to.
 template <typename R> static hs_status fft_prepare_t(Plan* p) {
-    HS_TRY((launch_fft<R, -1, ROW_FWD>(p, nullptr, nullptr, 0, nullptr)));
-    HS_TRY((launch_fft<R, -1, COL_FWD>(p, nullptr, nullptr, 0, nullptr)));
-    HS_TRY((launch_fft<R, 1, COL_INV>(p, nullptr, nullptr, 0, nullptr)));
-    return launch_fft<R, 1, ROW_INV>(p, nullptr, nullptr, 0, nullptr);
+    HS_TRY((launch_fft<R, -1, ROW_FWD>(p, nullptr, nullptr, 0, 0, nullptr)));
+    HS_TRY((launch_fft<R, -1, COL_FWD>(p, nullptr, nullptr, 0, 0, nullptr)));
+    HS_TRY((launch_fft<R, 1, COL_INV>(p, nullptr, nullptr, 0, 0, nullptr)));
+    return launch_fft<R, 1, ROW_INV>(p, nullptr, nullptr, 0, 0, nullptr);
 }
 hs_status fft_prepare(Plan* p) {
     if (!p->half) return plane_fft_init();
@@ -469,11 +478,11 @@ hs_status fft_forward(Plan* p, const void* X, cudaStream_t s) {
     if (!p->half) return plane_fft_forward(p, X, s);
     const int L = p->g.L;
     if (p->prec == HS_F32) {
-        HS_TRY((launch_fft<float, -1, ROW_FWD>(p, X, p->tmp, L, s)));
-        HS_TRY((launch_fft<float, -1, COL_FWD>(p, p->tmp, p->grid, L, s)));
+        HS_TRY((launch_fft<float, -1, ROW_FWD>(p, X, p->tmp, 0, L, s)));
+        HS_TRY((launch_fft<float, -1, COL_FWD>(p, p->tmp, p->grid, 0, L, s)));
     } else {
-        HS_TRY((launch_fft<double, -1, ROW_FWD>(p, X, p->tmp, L, s)));
-        HS_TRY((launch_fft<double, -1, COL_FWD>(p, p->tmp, p->grid, L, s)));
+        HS_TRY((launch_fft<double, -1, ROW_FWD>(p, X, p->tmp, 0, L, s)));
+        HS_TRY((launch_fft<double, -1, COL_FWD>(p, p->tmp, p->grid, 0, L, s)));
     }
     return HS_OK;
 }
@@ -499,14 +508,14 @@ template <typename R> static hs_status fft_adjoint_t(Plan* p, R* X, cudaStream_t
         const int n = std::min(C, L - l0);
         const Cx<R>* g = (const Cx<R>*)p->grid + l0 * gch;
         Cx<R>* t = (Cx<R>*)p->tmp + l0 * tch;
-        if (p->half) HS_TRY((launch_fft<R, 1, COL_INV>(p, g, t, n, s)));
-        else HS_TRY(plane_fft_cols_inv(p, g, t, n, s));
+        if (p->half) HS_TRY((launch_fft<R, 1, COL_INV>(p, g, t, l0, n, s)));
+        else HS_TRY(plane_fft_cols_inv(p, g, t, l0, n, s));
         if (side) {
             HS_CHECK_CUDA(cudaEventRecord(p->fft_ev_col, s));
             HS_CHECK_CUDA(cudaStreamWaitEvent(s2, p->fft_ev_col, 0));
         }
-        if (p->half) HS_TRY((launch_fft<R, 1, ROW_INV>(p, t, X + l0 * xch, n, s2)));
-        else HS_TRY(plane_fft_rows_inv(p, t, X + l0 * xch, n, s2));
+        if (p->half) HS_TRY((launch_fft<R, 1, ROW_INV>(p, t, X + l0 * xch, l0, n, s2)));
+        else HS_TRY(plane_fft_rows_inv(p, t, X + l0 * xch, l0, n, s2));
     }
     if (side) {
         HS_CHECK_CUDA(cudaEventRecord(p->fft_ev_join, s2));

@@ -44,6 +44,7 @@ template <typename R> struct FftArgs {
     int lgK, lgG;      // log2 K, log2 G
     int nx, ny, Kx, Ky;
     int lgny, lgKx;    // log2 ny, log2 Kx
+    const int4* rng;   // cells reached, per channel (the rest of the plane is never read)
 };
 
 // A line is a row (l, iy) of the row modes or a column (l, kx) of the column
@@ -78,8 +79,10 @@ __device__ __forceinline__ Cx<R> fft_load(const FftArgs<R>& a, int la, int lb, i
         else return cx<R>(0, 0);
         return ((const CT*)a.in)[((int64_t)la * a.ny + iy) * a.Kx + lb];
     } else if (MODE == COL_INV) {
+        if (!row_reached(a.rng[la], k)) return cx<R>(0, 0);
         return ((const CT*)a.in)[((int64_t)la * a.Ky + k) * a.Kx + lb];
     } else {   // ROW_INV
+        if (!col_reached(a.rng[la], k)) return cx<R>(0, 0);
         return ((const CT*)a.in)[((int64_t)la * a.ny + lb) * a.Kx + k];
     }
 }
@@ -88,9 +91,9 @@ template <typename R, int MODE>
 __device__ __forceinline__ void fft_store(const FftArgs<R>& a, int la, int lb, int k, Cx<R> v) {
     typedef Cx<R> CT;
     if (MODE == ROW_FWD) {
-        ((CT*)a.out)[((int64_t)la * a.ny + lb) * a.Kx + k] = v;
+        if (col_reached(a.rng[la], k)) ((CT*)a.out)[((int64_t)la * a.ny + lb) * a.Kx + k] = v;
     } else if (MODE == COL_FWD) {
-        ((CT*)a.out)[((int64_t)la * a.Ky + k) * a.Kx + lb] = v;
+        if (row_reached(a.rng[la], k)) ((CT*)a.out)[((int64_t)la * a.Ky + k) * a.Kx + lb] = v;
     } else if (MODE == COL_INV) {   // keep the ny image rows
         const int h = a.ny >> 1;
         int iy;
@@ -198,6 +201,13 @@ __device__ __forceinline__ void fft_pass(const FftArgs<R>& a, Cx<R>* sm, int lgN
     __syncthreads();
 }
 
+// A column group (at most 8 columns from a multiple of their number) that no window reaches.
+template <typename R, int MODE> __device__ __forceinline__ bool unreached(const FftArgs<R>& a, int line0) {
+    if (MODE != COL_FWD && MODE != COL_INV) return false;
+    const int la = line0 / a.Kx, c = line0 - la * a.Kx;
+    return !col_reached(a.rng[la], c) && !col_reached(a.rng[la], c + a.G - 1);
+}
+
 // DIR = -1: forward transform (exp(-2 pi i kn / K)); DIR = +1: unnormalised inverse.
 // LGK_ > 0: K = 2^LGK_ lines of G = 2^LGG_ per CTA fixed at compile time (the
 // pass schedule and every index computation fold to constants); 0: generic.
@@ -208,6 +218,7 @@ __global__ void __launch_bounds__(512, NREP > 1 ? 1 : (sizeof(R) == 4 ? 3 : 2)) 
     if constexpr (LGK_ > 0) {
         constexpr int N8 = LGK_ / 3, REM = LGK_ % 3, NPASS = N8 + (REM ? 1 : 0);
         const int line0 = blockIdx.x << LGG_;
+        if (unreached<R, MODE>(a, line0)) return;
 #pragma unroll
         for (int pass = 0; pass < NPASS; ++pass) {
             const bool first = (pass == 0), last = (pass == NPASS - 1);
@@ -217,6 +228,7 @@ __global__ void __launch_bounds__(512, NREP > 1 ? 1 : (sizeof(R) == 4 ? 3 : 2)) 
         }
     } else {
         const int line0 = blockIdx.x * a.G;
+        if (unreached<R, MODE>(a, line0)) return;
         int lgNs = 0;
         for (int pass = 0; pass < a.npass; ++pass) {
             const bool first = (pass == 0), last = (pass == a.npass - 1);
@@ -268,6 +280,7 @@ __global__ void __launch_bounds__(512) k_plane_fft_mr(FftArgs<R> a, MrPlan mp) {
     CT* src = reinterpret_cast<CT*>(smem_raw);
     CT* dst = src + GK;
     const int line0 = blockIdx.x * G, tid = threadIdx.x, nthr = blockDim.x;
+    if (unreached<R, MODE>(a, line0)) return;
     for (int e = tid; e < GK; e += nthr) {   // consecutive threads: consecutive columns / row elements
         const int g = COLS ? e % G : e / K, k = COLS ? e / G : e % K;
         int la, lb;
@@ -354,9 +367,9 @@ static void radix_plan(int K, int* n8, int* rlast, int* npass) {
     *npass = *n8 + (rem ? 1 : 0);
 }
 
-// nl channels starting at in / out (a channel range of the plan's cube).
+// nl channels from l0, starting at in / out (a channel range of the plan's cube).
 template <typename R, int DIR, int MODE>
-static hs_status launch_fft(Plan* p, const void* in, void* out, int nl, cudaStream_t s) {
+static hs_status launch_fft(Plan* p, const void* in, void* out, int l0, int nl, cudaStream_t s) {
     FftArgs<R> a;
     a.in = in;
     a.out = out;
@@ -364,6 +377,7 @@ static hs_status launch_fft(Plan* p, const void* in, void* out, int nl, cudaStre
     a.ny = p->g.ny;
     a.Kx = p->g.Kx;
     a.Ky = p->g.Ky;
+    a.rng = p->rng + l0;
     a.cxs = (const R*)p->cxs;
     a.cys = (const R*)p->cys;
     constexpr bool cols = (MODE == COL_FWD || MODE == COL_INV);
@@ -497,16 +511,16 @@ hs_status plane_fft_init() {
 }
 
 hs_status plane_fft_forward(Plan* p, const void* X, cudaStream_t s) {
-    HS_TRY((launch_fft<float, -1, ROW_FWD>(p, X, p->tmp, p->g.L, s)));
-    return launch_fft<float, -1, COL_FWD>(p, p->tmp, p->grid, p->g.L, s);
+    HS_TRY((launch_fft<float, -1, ROW_FWD>(p, X, p->tmp, 0, p->g.L, s)));
+    return launch_fft<float, -1, COL_FWD>(p, p->tmp, p->grid, 0, p->g.L, s);
 }
 
-hs_status plane_fft_cols_inv(Plan* p, const void* grid, void* tmp, int nl, cudaStream_t s) {
-    return launch_fft<float, 1, COL_INV>(p, grid, tmp, nl, s);
+hs_status plane_fft_cols_inv(Plan* p, const void* grid, void* tmp, int l0, int nl, cudaStream_t s) {
+    return launch_fft<float, 1, COL_INV>(p, grid, tmp, l0, nl, s);
 }
 
-hs_status plane_fft_rows_inv(Plan* p, const void* tmp, void* X, int nl, cudaStream_t s) {
-    return launch_fft<float, 1, ROW_INV>(p, tmp, X, nl, s);
+hs_status plane_fft_rows_inv(Plan* p, const void* tmp, void* X, int l0, int nl, cudaStream_t s) {
+    return launch_fft<float, 1, ROW_INV>(p, tmp, X, l0, nl, s);
 }
 
 }  // namespace hs

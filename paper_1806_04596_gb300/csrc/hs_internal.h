@@ -78,6 +78,14 @@ struct Coord64 {
 // 31 of the plan's permutation marks them.
 constexpr unsigned PERM_MIRROR = 0x80000000u;
 
+// Cells of one channel's grid that its windows reach, as an int4: columns c < x or
+// c >= y (multiples of 8), rows k < z or k >= w (both lie around frequency 0). The
+// coverage scales with the channel's frequency, so the lower channels of an octave use
+// about half of each axis: the other columns are neither transformed nor stored, and
+// rows outside are neither stored nor read. Gridding writes every cell inside.
+__host__ __device__ __forceinline__ bool col_reached(const int4& r, int c) { return c < r.x || c >= r.y; }
+__host__ __device__ __forceinline__ bool row_reached(const int4& r, int k) { return k < r.z || k >= r.w; }
+
 // Sizes passed by value to kernels.
 struct Geo {
     int nx, ny, L, Kx, Ky;
@@ -144,6 +152,8 @@ struct Plan {
     void* twy = nullptr;               // Ky complex
     void* filt = nullptr;              // 8 * 2 * MAXF reals: lowpass, highpass per db_p
     // scratch
+    int4* rng = nullptr;               // per channel: the cells its windows reach (Reach below)
+    std::vector<int4> rng_h;           // the same on the host
     void* grid = nullptr;              // L * Ky * Kw complex
     void* tmp = nullptr;               // L * ny * Kc complex
     void* vis = nullptr;               // M_total complex (sorted order)
@@ -190,8 +200,8 @@ struct Plan {
 hs_status plane_plan(Plan* p, std::shared_ptr<Plan>* out, cudaStream_t s);
 // FFT of the whole plane (hs_fft_plane.cu; FP32).
 hs_status plane_fft_forward(Plan* p, const void* X, cudaStream_t s);
-hs_status plane_fft_cols_inv(Plan* p, const void* grid, void* tmp, int nl, cudaStream_t s);
-hs_status plane_fft_rows_inv(Plan* p, const void* tmp, void* X, int nl, cudaStream_t s);
+hs_status plane_fft_cols_inv(Plan* p, const void* grid, void* tmp, int l0, int nl, cudaStream_t s);
+hs_status plane_fft_rows_inv(Plan* p, const void* tmp, void* X, int l0, int nl, cudaStream_t s);
 hs_status plane_fft_init();
 
 // Device allocation tracked by the plan (freed in destroy).

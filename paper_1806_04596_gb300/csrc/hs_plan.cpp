@@ -319,6 +319,14 @@ static hs_status build_sweep(Plan* p) {
     std::vector<int> ent;
     HS_TRY(sweep_lists(Kx, Ky, p->g.L, p->off_h.data(), p->k0x_h.data(), p->k0y_h.data(), p->sw_rows,
                        p->sw_cap, items, ent));
+    if (p->half) {   // cells that no window of the channel reaches are never read
+        auto unread = [&](const SweepItem& it) {
+            const int4 r = p->rng_h[it.l];
+            const int c0 = it.strip * GRID_TILE;
+            return (c0 >= r.x && c0 + GRID_TILE <= r.y) || (it.row0 >= r.z && it.row1 <= r.w);
+        };
+        items.erase(std::remove_if(items.begin(), items.end(), unread), items.end());
+    }
     if (p->sw_items) {   // rebuilt by the autotuner: replace the previous lists
         plan_release(p, p->sw_items);
         plan_release(p, p->sw_ent);
@@ -639,6 +647,23 @@ static hs_status build_layout(Plan* p, const std::vector<double>& uvh, const std
         }
         HS_TRY(upload(p, &p->coords, c));
     }
+    // cells that each channel's windows reach, from the stored start cells
+    p->rng_h.resize(L);
+    parallel_for(L, M, [&](int l) {
+        int xmax = 0, xmin = 0, ymax = 0, ymin = 0;   // [xmin, xmax) around frequency 0
+        for (int64_t i = p->off_h[l]; i < p->off_h[l + 1]; ++i) {
+            const int x = cellx[i], y = modk(celly[i] - 3, Ky);
+            const int sx = (!p->half && x >= Kx / 2) ? x - Kx : x, sy = y >= Ky / 2 ? y - Ky : y;
+            xmax = std::max(xmax, sx + 8);
+            xmin = std::min(xmin, sx);
+            ymax = std::max(ymax, sy + 8);
+            ymin = std::min(ymin, sy);
+        }
+        const int ncol = p->half ? g.Kw : Kx;
+        p->rng_h[l] = {std::min((xmax + 7) / 8 * 8, ncol), xmin < 0 ? (ncol + xmin) / 8 * 8 : ncol,
+                       std::min(ymax, Ky), Ky + ymin};
+    });
+    HS_TRY(upload(p, (void**)&p->rng, p->rng_h));
     if (!wh.empty()) {
         std::vector<double> ws(M);
         for (int64_t r = 0; r < M; ++r) ws[r] = wh[perm[r]];
