@@ -191,7 +191,7 @@ struct Plan {
     size_t csize() const { return 2 * rsize(); }
 };
 
-// The whole-plane layout of an FP32 plan's coverage (grid, lists, scratch of its own), built on
+// The whole-plane layout of an FP32 plan's coverage (lists of its own, the plan's scratch), built on
 // the first call and shared while a state holds it. The iteration with the nuclear prior uses
 // it: its eigensolver, warm-started with at most one Jacobi sweep per iteration, turns last-bit
 // differences of the gradient into 1e-4 of the image over the first ten iterations (256 x 256,

@@ -389,33 +389,35 @@ static hs_status time_ms(cudaStream_t s, int reps, const std::function<hs_status
     return st;
 }
 
+static TuneKey tune_key(const Plan* p) {
+    return {p->g.Kx, p->g.Ky, p->g.L, (int)p->prec, p->flags | (p->half ? 0u : 0x80000000u), p->M_total};
+}
+
+// Choices of an earlier plan of the same shape, before the lists are built (they are
+// then built once).
+static void take_tuned(Plan* p) {
+    if (p->flags & HS_PLAN_NO_TUNE) return;
+    std::lock_guard<std::mutex> lock(g_tune_mu);
+    auto it = g_tune_cache.find(tune_key(p));
+    if (it == g_tune_cache.end()) return;
+    const TuneVal& v = it->second;
+    p->gram_tc = v.gram_tc;
+    p->fft_adj_chunk = v.fft_chunk;
+    p->sweep_hmax = v.hmax;
+    p->sweep_cap = v.cap;
+    p->sw_rows = v.rows;
+    p->sw_cap = v.rcap;
+    p->sw_coop = v.coop;
+    std::copy(v.grid_ms, v.grid_ms + 3, p->tune_grid_ms);
+    std::copy(v.gram_ms, v.gram_ms + 2, p->tune_gram_ms);
+    std::copy(v.fft_ms, v.fft_ms + 2, p->tune_fft_ms);
+    p->tuned = 2;
+}
+
 static hs_status autotune(Plan* p, cudaStream_t s) {
     const auto t0 = std::chrono::steady_clock::now();
     const bool sweep = sweep_grid(p);
-    const TuneKey key{p->g.Kx, p->g.Ky, p->g.L, (int)p->prec, p->flags | (p->half ? 0u : 0x80000000u), p->M_total};
-    {
-        std::lock_guard<std::mutex> lock(g_tune_mu);
-        auto it = g_tune_cache.find(key);
-        if (it != g_tune_cache.end()) {
-            const TuneVal& v = it->second;
-            p->gram_tc = v.gram_tc;
-            p->fft_adj_chunk = v.fft_chunk;
-            std::copy(v.grid_ms, v.grid_ms + 3, p->tune_grid_ms);
-            std::copy(v.gram_ms, v.gram_ms + 2, p->tune_gram_ms);
-            std::copy(v.fft_ms, v.fft_ms + 2, p->tune_fft_ms);
-            p->sweep_hmax = v.hmax;
-            p->sweep_cap = v.cap;
-            p->sw_coop = v.coop;
-            if (sweep && (v.rows != p->sw_rows || v.rcap != p->sw_cap)) {
-                p->sw_rows = v.rows;
-                p->sw_cap = v.rcap;
-                HS_TRY(build_sweep(p));
-            }
-            p->tuned = 2;
-            p->tune_ms = std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t0).count();
-            return HS_OK;
-        }
-    }
+    if (p->tuned == 2) return HS_OK;   // taken from the cache
     const int L = p->g.L;
     const int64_t N = p->N();
     const int reps = 3;
@@ -487,7 +489,7 @@ static hs_status autotune(Plan* p, cudaStream_t s) {
         std::copy(p->tune_grid_ms, p->tune_grid_ms + 3, v.grid_ms);
         std::copy(p->tune_gram_ms, p->tune_gram_ms + 2, v.gram_ms);
         std::copy(p->tune_fft_ms, p->tune_fft_ms + 2, v.fft_ms);
-        g_tune_cache[key] = v;
+        g_tune_cache[tune_key(p)] = v;
     }
     p->tuned = 1;
     p->tune_ms = std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t0).count();
@@ -679,6 +681,7 @@ static hs_status build_layout(Plan* p, const std::vector<double>& uvh, const std
 
     // gridding lists: the sweep kernel's for grids of at least 64 x 64 cells;
     // per-tile lists for smaller grids and the compensated kernel
+    take_tuned(p);
     const bool sweep = sweep_grid(p);
     if (sweep) {
         p->k0x_h.resize(M);
@@ -850,14 +853,17 @@ static hs_status build_layout(Plan* p, const std::vector<double>& uvh, const std
         HS_TRY(upload_real<double>(p, &p->twy, twy));
     }
 
-    HS_TRY(plan_alloc(p, &p->grid, (size_t)L * Ky * g.Kw * p->csize()));
-    HS_TRY(plan_alloc(p, &p->tmp, (size_t)L * g.ny * g.Kc * p->csize()));
-    HS_TRY(plan_alloc(p, &p->vis, (size_t)std::max<int64_t>(M, 1) * p->csize()));
+    if (p->half) {   // the whole-plane layout of the same plan uses this scratch too (plane_plan)
+        const bool wide = p->prec == HS_F32 && L <= MAX_L_NUC;
+        HS_TRY(plan_alloc(p, &p->grid, (size_t)L * Ky * (wide ? Kx : g.Kw) * p->csize()));
+        HS_TRY(plan_alloc(p, &p->tmp, (size_t)L * g.ny * (wide ? Kx : g.Kc) * p->csize()));
+        HS_TRY(plan_alloc(p, &p->vis, (size_t)std::max<int64_t>(M, 1) * p->csize()));
+    }
     HS_CHECK_CUDA(cudaStreamCreateWithFlags(&p->fft_side, cudaStreamNonBlocking));
     HS_CHECK_CUDA(cudaEventCreateWithFlags(&p->fft_ev_col, cudaEventDisableTiming));
     HS_CHECK_CUDA(cudaEventCreateWithFlags(&p->fft_ev_join, cudaEventDisableTiming));
     HS_TRY(fft_prepare(p));
-    if (p->flags & HS_PLAN_FFT_CHUNKED) p->fft_adj_chunk = fft_adjoint_chunk(p);
+    if ((p->flags & HS_PLAN_FFT_CHUNKED) && p->tuned != 2) p->fft_adj_chunk = fft_adjoint_chunk(p);
     return HS_OK;
 }
 
@@ -1001,7 +1007,9 @@ hs_status plan_create(Plan** out, int nx, int ny, int L, const int64_t* vis_offs
 }
 
 // The whole-plane companion of an FP32 plan: same coverage, blocks, weights and
-// flags; p stays unchanged but for the shared reference.
+// flags, lists and coordinates of its own, the plan's grid scratch (as the plan's own calls
+// and every state on it use that, in stream order); p stays unchanged but for the
+// shared reference.
 hs_status plane_plan(Plan* p, std::shared_ptr<Plan>* out, cudaStream_t s) {
     std::lock_guard<std::mutex> lock(p->plane_mu);
     *out = p->plane.lock();
@@ -1043,16 +1051,31 @@ hs_status plane_plan(Plan* p, std::shared_ptr<Plan>* out, cudaStream_t s) {
         HS_TRY(unsorted(p->u_sorted, uh));
     }
     HS_TRY(build_layout(c.get(), uvh, wh, uh, s));
-    if (!(c->flags & HS_PLAN_NO_TUNE)) {   // F^H candidates write a cube that only the tuning needs
-        const size_t bytes = (size_t)c->g.L * c->N() * c->rsize();
-        HS_TRY(lib_alloc(&c->xbuf, bytes));
-        const hs_status e = autotune(c.get(), s);
-        const cudaError_t ce = cudaStreamSynchronize(s);
-        lib_free(c->xbuf, bytes);
+    if (!(c->flags & HS_PLAN_NO_TUNE) && c->tuned == 0) {
+        // the candidates run on scratch of their own: another state may be iterating on the plan's.
+        // Without room for it the layout keeps the default choices.
+        const size_t bytes[4] = {(size_t)c->g.L * c->g.Ky * c->g.Kw * c->csize(),
+                                 (size_t)c->g.L * c->g.ny * c->g.Kc * c->csize(),
+                                 (size_t)std::max<int64_t>(M, 1) * c->csize(), (size_t)c->g.L * c->N() * c->rsize()};
+        void** const buf[4] = {&c->grid, &c->tmp, &c->vis, &c->xbuf};
+        int got = 0;
+        while (got < 4 && lib_alloc(buf[got], bytes[got]) == HS_OK) ++got;
+        hs_status e = HS_OK;
+        cudaError_t ce = cudaSuccess;
+        if (got == 4) {
+            e = autotune(c.get(), s);
+            ce = cudaStreamSynchronize(s);
+        } else {
+            clear_error();
+        }
+        for (int k = 0; k < got; ++k) lib_free(*buf[k], bytes[k]);
         c->xbuf = nullptr;
         HS_TRY(e);
         HS_CHECK_CUDA(ce);
     }
+    c->grid = p->grid;
+    c->tmp = p->tmp;
+    c->vis = p->vis;
     c->k0x_h.clear();
     c->k0y_h.clear();
     c->k0x_h.shrink_to_fit();
