@@ -44,6 +44,7 @@ constexpr int KB_HALF = 7;           // even (or odd) coefficients of a piece, a
 constexpr int GRID_TILE = 32;        // gridding tile side (cells)
 constexpr int GRID_WARPS = 4;        // warps per gridding CTA (private accumulators)
 constexpr int GRID_CAP = 512;        // most list entries one gridding CTA processes
+constexpr int64_t TAPS_MAX = (int64_t)2 << 30;   // most bytes of FP64 tap tables (16.8M visibilities)
 constexpr int DEGRID_CHUNK = 256;    // visibilities per degridding CTA
 constexpr int SWEEP_HMAX = 64;       // most output rows of one sweep-gridding work item
 constexpr int SWEEP_CAP = 1024;      // windows above which a sweep item's rows are cut short
@@ -123,6 +124,7 @@ struct Plan {
     int64_t* off_d = nullptr;          // L+1
     int* perm = nullptr;               // sorted index -> caller index (PERM_MIRROR: value conjugated)
     void* coords = nullptr;            // FP32: uint2 fixed point; FP64: Coord64
+    void* taps = nullptr;              // FP64 plans: 16 kernel taps per visibility (up to TAPS_MAX bytes)
     void* w_sorted = nullptr;          // Theta in sorted order (real) or null
     void* u_sorted = nullptr;          // U in sorted order (real) or null
     int64_t n_ent = 0;
@@ -258,6 +260,7 @@ struct GridArgs {
     void* v;                // GIN_PD: dual output v (home tile writes), sorted
 };
 hs_status grid(Plan* p, const GridArgs& a, cudaStream_t s);
+hs_status nufft_taps(Plan* p, cudaStream_t s);   // fills p->taps from the coordinates (FP64)
 
 // l2-ball helpers (hs_prox.cu)
 struct AdaptArgs {          // Algorithm 2 steps 13-19 on the device

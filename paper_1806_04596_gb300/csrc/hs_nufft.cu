@@ -23,6 +23,8 @@
 // shared memory, the copies combined in a fixed order. HS_PLAN_COMPENSATED
 // kernel: the same tiles, one window per warp at a time, with Kahan-compensated
 // FP32 sums.
+#include <algorithm>
+
 #include "hs_device.cuh"
 #include "hs_internal.h"
 
@@ -85,6 +87,7 @@ template <typename R> struct NufftK {
     const R* scale;
     const int64_t* tile_off;
     const int* tile_ent;
+    const R* taps;     // FP64: the 16 kernel taps of every sorted visibility, or null (Plan::taps)
     const int* blk;    // block of every sorted visibility (data blocks), or null: one block per channel
     double* rpart;     // DOUT_PD: per-item partial ||y - Phi x~||^2 (adaptive bounds), or null
 };
@@ -111,7 +114,7 @@ template <typename R> __device__ __forceinline__ void cp_async_cx(Cx<R>* dst, co
         asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(d), "l"(src) : "memory");
 }
 
-template <typename R, int NC, int MODE>
+template <typename R, int NC, int MODE, bool TAPS>
 __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 5 : 1)
     k_degrid(NufftK<R> a, const DgItem* __restrict__ items) {
     typedef Cx<R> CT;
@@ -146,10 +149,20 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 5 : 1)
     const int j = lane & 7;              // window column / tap owned by this lane
     const int grp = threadIdx.x >> 3;    // 32 groups of 8 lanes
     const int gbase = lane & ~7;
-    R c[NC];
-#pragma unroll
-    for (int k = 0; k < NC; ++k) c[k] = a.kbc[(7 - j) * NC + k];
     const int64_t beg = it.e0, end = it.e1;
+    R c[NC];           // the lane's kernel piece, or
+    R tu[8], tv[8];    // TAPS: its column and row taps of the group's 8 visibilities
+    if constexpr (TAPS) {
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            const int64_t i = beg + grp + 32 * k;
+            tu[k] = i < end ? a.taps[16 * i + j] : (R)0;
+            tv[k] = i < end ? a.taps[16 * i + 8 + j] : (R)0;
+        }
+    } else {
+#pragma unroll
+        for (int k = 0; k < NC; ++k) c[k] = a.kbc[(7 - j) * NC + k];
+    }
     R sq = 0;   // this thread's share of ||d||^2 (few terms; FP64 only for the block sum)
     R rq = 0;   // and of ||y - Phi x~||^2 (adaptive bounds)
     // lane j of a group preloads the coordinates of the group's j-th visibility
@@ -185,8 +198,13 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 5 : 1)
             const int ox = wrapn(cxv - tx0, Kw, kwm);
             const int oy = wrapn(wrapn(cyv - 3, Ky, kym) - ty0, Ky, kym);
             off[h] = min(oy, DG_REG - 8) * DG_LDS + min(ox, DG_REG - 8) + j;
-            pu[h] = horner<R, NC>(c, (R)2 * fx - (R)1);
-            pv[h] = horner<R, NC>(c, (R)2 * fy - (R)1);
+            if constexpr (TAPS) {
+                pu[h] = tu[it2 + h];
+                pv[h] = tv[it2 + h];
+            } else {
+                pu[h] = horner<R, NC>(c, (R)2 * fx - (R)1);
+                pv[h] = horner<R, NC>(c, (R)2 * fy - (R)1);
+            }
         }
         CT gv[2][8];
 #pragma unroll
@@ -735,9 +753,21 @@ __global__ void __launch_bounds__(COOP ? SW_COOP_MAX * 32 : SW_WARPS * 32, sizeo
                 if (rx >= 0 && ry >= 0 && ry < H) a.v[i] = val;
             }
             if (a.w) val = cscale(val, r.w);
-            R pu[8], pv[8];
-            taps((R)2 * fx - (R)1, pu);   // phi_u of window columns 0 .. 7
-            taps((R)2 * fy - (R)1, pv);   // phi_v of window rows 0 .. 7
+            R pu[8], pv[8];   // phi_u of window columns 0 .. 7, phi_v of window rows 0 .. 7
+            if (sizeof(R) == 8 && a.taps) {
+                const CT* tp = reinterpret_cast<const CT*>(a.taps + 16 * (int64_t)i);
+#pragma unroll
+                for (int m = 0; m < 4; ++m) {
+                    const CT u2 = tp[m], v2 = tp[4 + m];
+                    pu[2 * m] = u2.x;
+                    pu[2 * m + 1] = u2.y;
+                    pv[2 * m] = v2.x;
+                    pv[2 * m + 1] = v2.y;
+                }
+            } else {
+                taps((R)2 * fx - (R)1, pu);
+                taps((R)2 * fy - (R)1, pv);
+            }
 #pragma unroll
             for (int k = 0; k < 3 * (int)sizeof(R) / 4; ++k)   // 12 reals
                 reinterpret_cast<float4*>(rt)[k] = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -819,6 +849,39 @@ __global__ void k_grid_merge(const GridMerge* __restrict__ merges, const Cx<R>* 
     }
 }
 
+// Kernel taps of every sorted visibility of an FP64 plan, once at its creation: one thread
+// per visibility and axis, mirrored pieces as E(s^2) +- s O(s^2). An FP64 multiply-add costs
+// 64 FP32 ones, and the taps were most of what de-gridding (26 per lane and visibility)
+// and the sweep's decoding (112 per list entry, 1.5 to 2 entries per visibility) did.
+// us, before -> after: 128 x 128, L = 6, 9000 per channel de-gridding 55 -> 27, gridding 215 -> 137;
+// 64 x 64, L = 4 29 -> 15 and 168 -> 109.
+__global__ void k_taps64(const Coord64* __restrict__ c, int64_t n, const double* __restrict__ kbc,
+                         double* __restrict__ out) {
+    constexpr int NC = KB_TERMS_F64;
+    for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < 2 * n; t += (int64_t)gridDim.x * blockDim.x) {
+        const Coord64 q = c[t >> 1];
+        const double s = 2.0 * ((t & 1) ? q.fy : q.fx) - 1.0, s2 = s * s;
+        for (int m = 0; m < 4; ++m) {
+            const double* k = kbc + (7 - m) * NC;
+            double e = k[NC - 2], o = k[NC - 1];
+            for (int j = NC - 4; j >= 0; j -= 2) {
+                e = fma(e, s2, k[j]);
+                o = fma(o, s2, k[j + 1]);
+            }
+            out[8 * t + m] = fma(s, o, e);
+            out[8 * t + 7 - m] = fma(-s, o, e);
+        }
+    }
+}
+static_assert(KB_TERMS_F64 % 2 == 0, "even and odd coefficients in pairs");
+
+hs_status nufft_taps(Plan* p, cudaStream_t s) {
+    const unsigned nb = (unsigned)std::min<int64_t>((2 * p->M_total + 127) / 128, 8192);
+    k_taps64<<<nb, 128, 0, s>>>((const Coord64*)p->coords, p->M_total, (const double*)p->kbc, (double*)p->taps);
+    HS_CHECK_LAUNCH();
+    return HS_OK;
+}
+
 // ---------------------------------------------------------------- launches
 int degrid_blocks_x(const Plan* p) { return (p->Mmax + DEGRID_CHUNK - 1) / DEGRID_CHUNK; }
 int degrid_items_max(const Plan* p) { return p->dg_items_max > 0 ? p->dg_items_max : 1; }
@@ -843,6 +906,7 @@ template <typename R> static NufftK<R> base_args(Plan* p) {
         }
     k.tile_off = p->tile_off;
     k.tile_ent = p->tile_ent;
+    k.taps = sizeof(R) == 8 ? (const R*)p->taps : nullptr;
     k.blk = p->blk_id;
     k.nblk_x = degrid_blocks_x(p);
     return k;
@@ -861,13 +925,20 @@ static hs_status degrid_t(Plan* p, const DegridArgs& da, cudaStream_t s) {
     const unsigned nb = (unsigned)p->n_dg_items;
     const size_t sm = (size_t)DG_REG * DG_LDS * sizeof(Cx<R>);
     const DgItem* items = (const DgItem*)p->dg_items;
+    const bool taps = sizeof(R) == 8 && k.taps != nullptr;
+#define HS_DEGRID(MODE)                                                                       \
+    case MODE:                                                                                \
+        if (taps) k_degrid<R, NC, MODE, sizeof(R) == 8><<<nb, 256, sm, s>>>(k, items);        \
+        else k_degrid<R, NC, MODE, false><<<nb, 256, sm, s>>>(k, items);                      \
+        break
     switch (da.mode) {
-        case DOUT_CALLER: k_degrid<R, NC, DOUT_CALLER><<<nb, 256, sm, s>>>(k, items); break;
-        case DOUT_SORTED: k_degrid<R, NC, DOUT_SORTED><<<nb, 256, sm, s>>>(k, items); break;
-        case DOUT_SORTED_U: k_degrid<R, NC, DOUT_SORTED_U><<<nb, 256, sm, s>>>(k, items); break;
-        case DOUT_PD: k_degrid<R, NC, DOUT_PD><<<nb, 256, sm, s>>>(k, items); break;
+        HS_DEGRID(DOUT_CALLER);
+        HS_DEGRID(DOUT_SORTED);
+        HS_DEGRID(DOUT_SORTED_U);
+        HS_DEGRID(DOUT_PD);
         default: return fail(HS_ERR_ARG, "degrid: bad mode");
     }
+#undef HS_DEGRID
     HS_CHECK_LAUNCH();
     return HS_OK;
 }

@@ -939,6 +939,10 @@ static hs_status build(Plan* p, const int64_t* vis_offsets, int nblocks, const i
     HS_TRY(plan_alloc(p, (void**)&p->dscal, sizeof(double) * 6 * std::max(L, 1)));
     HS_TRY(plan_alloc(p, (void**)&p->err_d, sizeof(int)));
     HS_CHECK_CUDA(cudaMemsetAsync(p->err_d, 0, sizeof(int), s));
+    if (p->prec == HS_F64 && M > 0 && 16 * 8 * M <= TAPS_MAX) {   // optional: without room the taps are evaluated
+        if (plan_alloc(p, &p->taps, (size_t)M * 16 * sizeof(double)) == HS_OK) HS_TRY(nufft_taps(p, s));
+        else clear_error();
+    }
     if (p->flags & HS_PLAN_GRAM_FMA) p->gram_tc = 0;
     if (!(p->flags & HS_PLAN_NO_TUNE)) HS_TRY(autotune(p, s));
     p->k0x_h.clear();
