@@ -2,6 +2,7 @@
 // lifetime, operator entry points and the primal-dual iteration (Algorithm 2).
 #include <cmath>
 #include <cstring>
+#include <exception>
 #include <memory>
 #include <vector>
 
@@ -131,8 +132,12 @@ hs_status hs_sweep_lists(int Kx, int Ky, int L, const int64_t* offsets, const in
             return fail(HS_ERR_ARG, "hs_sweep_lists: start cell %lld outside the grid", (long long)r);
     std::vector<hs::SweepItem> it;
     std::vector<int> en;
-    HS_TRY(hs::sweep_lists(Kx, Ky, L, offsets, k0x, k0y, hmax > 0 ? hmax : hs::SWEEP_HMAX,
-                           cap > 0 ? cap : hs::SWEEP_CAP, it, en));
+    try {
+        HS_TRY(hs::sweep_lists(Kx, Ky, L, offsets, k0x, k0y, hmax > 0 ? hmax : hs::SWEEP_HMAX,
+                               cap > 0 ? cap : hs::SWEEP_CAP, it, en));
+    } catch (const std::exception& e) {
+        return fail(HS_ERR_NOMEM, "hs_sweep_lists: host allocation failed: %s", e.what());
+    }
     if (items != nullptr && ent != nullptr) {
         if (*n_items < (int64_t)it.size() || *n_ent < (int64_t)en.size())
             return fail(HS_ERR_ARG, "hs_sweep_lists: buffers hold %lld items / %lld entries, need %lld / %lld",

@@ -187,6 +187,15 @@ static void parallel_for(int n, int64_t items, const std::function<void(int)>& f
     if (err) std::rethrow_exception(err);
 }
 
+// f(), with host allocation failures as a status (no exception passes the C boundary).
+template <typename F> static hs_status no_throw(F f) {
+    try {
+        return f();
+    } catch (const std::exception& e) {
+        return fail(HS_ERR_NOMEM, "host allocation failed while building a plan: %s", e.what());
+    }
+}
+
 // Gridding lists of the sweep kernel (grids of at least 64 x 64 cells). A work
 // item is one channel, one 32-column strip and its output rows [row0, row1);
 // its list holds every window that overlaps the strip and starts in rows
@@ -1001,7 +1010,8 @@ hs_status plan_create(Plan** out, int nx, int ny, int L, const int64_t* vis_offs
     g.fbx = std::min(23, 32 - ilog2(g.Kx));
     g.fby = std::min(23, 32 - ilog2(g.Ky));
     g.kym = pow2(g.Ky) ? g.Ky - 1 : -1;
-    hs_status st = build(p.get(), vis_offsets, nblocks, block_offsets, uv, weights, precond, s);
+    const hs_status st =
+        no_throw([&]() { return build(p.get(), vis_offsets, nblocks, block_offsets, uv, weights, precond, s); });
     if (st != HS_OK) {
         plan_free(p.get());
         return st;
@@ -1014,7 +1024,12 @@ hs_status plan_create(Plan** out, int nx, int ny, int L, const int64_t* vis_offs
 // flags, lists and coordinates of its own, the plan's grid scratch (as the plan's own calls
 // and every state on it use that, in stream order); p stays unchanged but for the
 // shared reference.
+static hs_status make_plane(Plan* p, std::shared_ptr<Plan>* out, cudaStream_t s);
 hs_status plane_plan(Plan* p, std::shared_ptr<Plan>* out, cudaStream_t s) {
+    return no_throw([&]() { return make_plane(p, out, s); });
+}
+
+static hs_status make_plane(Plan* p, std::shared_ptr<Plan>* out, cudaStream_t s) {
     std::lock_guard<std::mutex> lock(p->plane_mu);
     *out = p->plane.lock();
     if (*out) return HS_OK;
@@ -1067,7 +1082,7 @@ hs_status plane_plan(Plan* p, std::shared_ptr<Plan>* out, cudaStream_t s) {
         hs_status e = HS_OK;
         cudaError_t ce = cudaSuccess;
         if (got == 4) {
-            e = autotune(c.get(), s);
+            e = no_throw([&]() { return autotune(c.get(), s); });
             ce = cudaStreamSynchronize(s);
         } else {
             clear_error();
