@@ -267,10 +267,10 @@ def job_rate(ms: float, steps: int, world: int, device: str = "cuda"):
 # Resource that limits each stage in practice (ncu: profiles/kernel_sections_c2.md,
 # profiles/stage_traffic.txt); the roofline each is measured against is HBM.
 LIMITER = {
-    "fft_fwd": "HBM: spectrum write plus the row-pass intermediate",
+    "fft_fwd": "latency and shared-memory exchanges of the radix passes (half-plane spectrum)",
     "degrid": "shared-memory data pipe and instruction issue (8 lanes per visibility, staged window rows)",
     "grid": "instruction issue and shared-memory data pipe (12 row taps per lane per window group)",
-    "fft_adj": "HBM: the row-pass intermediate round trip (1.57x algorithmic bytes)",
+    "fft_adj": "latency and shared-memory exchanges of the radix passes (half-plane spectrum)",
     "psi_fwd": "instruction issue of the first level (filter taps of 8 wavelets, staging, barriers)",
     "psi_adj": "instruction issue of the first level; instruction fetch in the shared-memory tail",
     "gram": "instruction issue (digit split and accumulator drain per 64-pixel chunk)",
