@@ -1222,12 +1222,18 @@ __global__ void __launch_bounds__(TAIL_THREADS) k_dwt_inv_tail(const R* __restri
 
 // First level of the shared-memory tail: the finest level lev >= 1 whose input
 // block fits (both sides multiples of 8 at every level down to the top), or 0
-// when no level qualifies.
+// when no level qualifies. FP64 tails are bound by the FP64 pipes of the SMs they sit on: while
+// one SM in six or more would have none, they start a level later, at 32 samples, and the
+// level before runs on tiles over the whole chip. 128 x 128, from 64 against from 32, analysis
+// and synthesis: 72 tails 123.0/139.1 and 106.6/125.5 us, 112 tails 176.2/192.6 and
+// 168.0/190.6; 256 x 256, 96 tails: 459.6/528.7 and 455.4/523.9. Above, one launch more costs
+// what the tiles gain: 256 x 128, 144 tails 317.2/361.8 and 319.4/367.0.
 template <typename R> static int tail_level(const Plan* p) {
     const int top = p->levels - 1;
+    const int widest = sizeof(R) == 8 && NW * p->g.L < 128 ? 32 : tail_max_width<R>();
     for (int lev = 1; lev <= top; ++lev) {
         const int my = p->g.ny >> lev, mx = p->g.nx >> lev;
-        if (mx > tail_max_width<R>() || tail_smem<R>(my) > (size_t)TAIL_SMEM_MAX) continue;
+        if (mx > widest || tail_smem<R>(my) > (size_t)TAIL_SMEM_MAX) continue;
         for (int j = lev; j <= top; ++j)
             if (((p->g.ny >> j) % 8) || ((p->g.nx >> j) % 8)) return 0;
         return lev;
