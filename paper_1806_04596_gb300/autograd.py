@@ -36,6 +36,9 @@ from . import hypersara as hs
 
 
 def _c(t):
+    """t as the kernels read it: contiguous, lazy conjugation and negation (which torch keeps as
+    a bit beside the memory, as in the gradient of z.conj()) written out."""
+    t = t.resolve_conj().resolve_neg()
     return t if t.is_contiguous() else t.contiguous()
 
 
