@@ -42,6 +42,16 @@ def _c(t):
     return t if t.is_contiguous() else t.contiguous()
 
 
+def _has_memory(t):
+    """False for tensors that stand for others (the batched gradients of is_grads_batched, vmap):
+    torch operations take them, a kernel cannot."""
+    try:
+        t.data_ptr()
+    except RuntimeError:
+        return False
+    return True
+
+
 class _Phi(torch.autograd.Function):
     @staticmethod
     def forward(ctx, X, plan):
@@ -97,7 +107,8 @@ class _L21Norm(torch.autograd.Function):
     @staticmethod
     def backward(ctx, g):
         (A,) = ctx.saved_tensors
-        if torch.is_grad_enabled():   # create_graph: keep the product with g differentiable
+        # create_graph: keep the product with g differentiable
+        if torch.is_grad_enabled() or not _has_memory(g):
             return ctx.plan.l21_grad(_c(A), ctx.w_rows) * g, None, None
         return ctx.plan.l21_grad(_c(A), ctx.w_rows, scale=_c(g)), None, None
 

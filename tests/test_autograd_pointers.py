@@ -1,5 +1,6 @@
 """Gradients that reach the kernels as bare pointers: what torch keeps beside the memory
-(the conjugate and the negative bit) has to be in the memory. A stand-in plan on
+(the conjugate and the negative bit) has to be in the memory, and a gradient that has no
+memory (a batched one) must not get there. A stand-in plan on
 the CPU reads every tensor the way the library does, from its address."""
 
 import ctypes
@@ -62,3 +63,17 @@ def test_conjugate_bit_of_the_incoming_gradient():
     (g,) = torch.autograd.grad(loss, X)
     want = (torch.tensor(plan.F.conj()) * w[:, None]).sum(0).real.reshape(3, 2, 2)
     torch.testing.assert_close(g, want, rtol=1e-13, atol=1e-13)
+
+
+@pytest.mark.parametrize("vmapped", [False, True])
+def test_batched_incoming_gradients(vmapped):
+    plan = _Plan()
+    A = torch.randn((9, 3, 2, 2), dtype=torch.float64, requires_grad=True)
+    f = hsg.l21_norm(plan, A)
+    (g1,) = torch.autograd.grad(f, A, retain_graph=True)
+    c = torch.tensor([1.0, 2.0, -3.0], dtype=torch.float64)
+    if vmapped:
+        g = torch.vmap(lambda v: torch.autograd.grad(f, A, v, retain_graph=True)[0])(c)
+    else:
+        (g,) = torch.autograd.grad(f, A, grad_outputs=c, is_grads_batched=True, retain_graph=True)
+    torch.testing.assert_close(g, c[:, None, None, None, None] * g1, rtol=1e-15, atol=0.0)
