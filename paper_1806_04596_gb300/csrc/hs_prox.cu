@@ -169,18 +169,18 @@ __device__ __forceinline__ void pair_add(float& hi, float& lo, float x) {
 // form below (386 us at 512 x 512, L = 32, now 62: 302 MB that stream in 45). Here a square is
 // a pair p + e, exact (e from the fused multiply-add), and pairs are added with the
 // error-free two-sum; the root is an FP32 value r rounded from a Newton step plus the
-// correction (s - r^2) / 2r (its own error below 2^-49 of r); rows are added in pairs
-// too, and FP64 only sees one pair per thread. A lane owns two neighbouring rows at a
+// correction (s - r^2) / 2r (its own error below 2^-49 of r). A lane owns two neighbouring rows at a
 // time and 16 of their channels are in flight (the 4-warp split of k_l21_split, with its
 // two barriers per tile, took 148 us here). Rows whose squares leave the range in which
 // p + e is exact (or are not finite) are summed again in FP64.
+// Rows and their weights meet in FP64: in FP32 pairs the products of a thread's rows (162 at
+// 2048 x 2048) left the range although each one was inside it, and the sum became NaN.
 __global__ void __launch_bounds__(256) k_l21_norm_pairs(const float* __restrict__ A,
                                                         const float* __restrict__ w_rows, int L, int64_t N,
                                                         double* __restrict__ part) {
     __shared__ double red[32];
     const int64_t Nh = N >> 1;
-    double acc = 0.0;               // rows outside the range
-    float ahi = 0.f, alo = 0.f;     // the others
+    double acc = 0.0;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < NB * Nh;
          i += (int64_t)gridDim.x * blockDim.x) {
         const int b = (int)(i / Nh);
@@ -209,14 +209,12 @@ __global__ void __launch_bounds__(256) k_l21_norm_pairs(const float* __restrict_
         for (int k = 0; k < 2; ++k) {
             const float s = hi[k];
             const float wr = w_rows ? w_rows[(int64_t)b * N + pix + k] : 1.f;
-            if (s >= 0x1p-85f && s <= 0x1p126f && fabsf(wr) <= 0x1p60f && (fabsf(wr) >= 0x1p-40f || wr == 0.f)) {
+            if (s >= 0x1p-85f && s <= 0x1p126f) {
                 const float y = rsqrtf(s), h = 0.5f * y;
                 float r = s * y;
                 r = fmaf(h, fmaf(-r, r, s), r);
                 const float c = h * (__fmaf_rn(-r, r, s) + lo[k]);   // root = r + c
-                const float p = __fmul_rn(r, wr);
-                alo = __fadd_rn(alo, fmaf(c, wr, __fmaf_rn(r, wr, -p)));
-                pair_add(ahi, alo, p);
+                acc = fma((double)r + (double)c, (double)wr, acc);
             } else if (mx[k] != 0.f || !(s == 0.f)) {
                 double d = 0.0;
                 for (int l = 0; l < L; ++l) {
@@ -229,7 +227,7 @@ __global__ void __launch_bounds__(256) k_l21_norm_pairs(const float* __restrict_
             }
         }
     }
-    acc = block_sum(acc + ((double)ahi + (double)alo), red);
+    acc = block_sum(acc, red);
     if (threadIdx.x == 0) part[blockIdx.x] = acc;
 }
 
