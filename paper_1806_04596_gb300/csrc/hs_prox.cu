@@ -157,36 +157,45 @@ __global__ void __launch_bounds__(128) k_l21_split(const float* __restrict__ A, 
     }
 }
 
-// (hi, lo) += x exactly up to the rounding of lo (Knuth's two-sum).
-__device__ __forceinline__ void pair_add(float& hi, float& lo, float x) {
-    const float s = __fadd_rn(hi, x), t = __fsub_rn(s, hi);
-    lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(s, t)), __fsub_rn(x, t)));
-    hi = s;
+// Knuth's two-sum: a + x exactly, as the rounded sum (left in a) and the returned rest.
+__device__ __forceinline__ float two_sum(float& a, float x) {
+    const float s = __fadd_rn(a, x), t = __fsub_rn(s, a);
+    const float e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, t)), __fsub_rn(x, t));
+    a = s;
+    return e;
 }
 
-// l2,1 norm of an FP32 cube in pairs of FP32 values. FP64 runs at 1/64 of the FP32
-// rate, and one conversion and one FP64 multiply-add per coefficient bounded the plain
-// form below (386 us at 512 x 512, L = 32, now 62: 302 MB that stream in 45). Here a square is
-// a pair p + e, exact (e from the fused multiply-add), and pairs are added with the
-// error-free two-sum; the root is an FP32 value r rounded from a Newton step plus the
-// correction (s - r^2) / 2r (its own error below 2^-49 of r). A lane owns two neighbouring rows at a
-// time and 16 of their channels are in flight (the 4-warp split of k_l21_split, with its
-// two barriers per tile, took 148 us here). Rows whose squares leave the range in which
-// p + e is exact (or are not finite) are summed again in FP64.
-// Rows and their weights meet in FP64: in FP32 pairs the products of a thread's rows (162 at
-// 2048 x 2048) left the range although each one was inside it, and the sum became NaN.
-__global__ void __launch_bounds__(256) k_l21_norm_pairs(const float* __restrict__ A,
+// l2,1 norm of an FP32 cube to FP64 accuracy, mostly in FP32: FP64 runs at 1/64 of the FP32
+// rate, and one conversion and one FP64 multiply-add per coefficient bound the plain form below.
+//  * A square is a pair p + e, exact (e from the fused multiply-add); p, e and the rest of p's
+//    addition are added with the error-free two-sum, and what two-sums leave over goes to
+//    a third value: ~68 bits of a row's sum s.
+//  * Its root is r + c + c2: r rounded, c the correction by the residual s - r^2, c2 by the
+//    residual of r + c (its own error below 2^-66 of r).
+//  * r times the weight is a pair again. Its high part goes to the FP64 sum (one conversion and one
+//    addition per row, where a root in FP64 took 17 instructions), its low part and the corrections to a
+//    pair that is added at the end.
+// With two values to a row and FP32 pairs for the rows the norm was 2 to 5e-16 off where the plain
+// form and this one are at 1e-16 and below; and the products of a thread's rows (162 at 2048 x 2048), each inside the FP32
+// range, left it together. A lane owns two neighbouring rows at a time and 16 of their channels
+// are in flight (the 4-warp split of k_l21_split, with its two barriers per tile, took 148 us at
+// 512 x 512, L = 32). Rows whose squares or products leave the range in which the pairs are exact
+// (or are not finite) are summed again in FP64. Bound by FP32 issue (24 instructions a coefficient):
+// us per call with the copy to the host, plain form -> two values -> this: 512 x 512, L = 32
+// 410 -> 87 -> 110; 1024 x 1024, L = 1 122 -> 183 for the last two (many rows of one channel).
+__global__ void __launch_bounds__(256) k_l21_norm_exact(const float* __restrict__ A,
                                                         const float* __restrict__ w_rows, int L, int64_t N,
                                                         double* __restrict__ part) {
     __shared__ double red[32];
     const int64_t Nh = N >> 1;
     double acc = 0.0;
+    float slo = 0.f, sll = 0.f;   // below acc: at most 2^-23 of what it holds
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < NB * Nh;
          i += (int64_t)gridDim.x * blockDim.x) {
         const int b = (int)(i / Nh);
         const int64_t pix = 2 * (i - (int64_t)b * Nh);
         const float* row = A + (int64_t)b * L * N + pix;
-        float hi[2] = {0.f, 0.f}, lo[2] = {0.f, 0.f}, mx[2] = {0.f, 0.f};
+        float hi[2] = {0.f, 0.f}, lo[2] = {0.f, 0.f}, ll[2] = {0.f, 0.f}, mx[2] = {0.f, 0.f};
         for (int l0 = 0; l0 < L; l0 += 16) {
             float2 v[16];
 #pragma unroll
@@ -199,8 +208,9 @@ __global__ void __launch_bounds__(256) k_l21_norm_pairs(const float* __restrict_
 #pragma unroll
                 for (int k = 0; k < 2; ++k) {
                     const float p = __fmul_rn(q[k], q[k]);
-                    lo[k] = __fadd_rn(lo[k], __fmaf_rn(q[k], q[k], -p));
-                    pair_add(hi[k], lo[k], p);
+                    const float e = two_sum(lo[k], __fmaf_rn(q[k], q[k], -p));
+                    const float f = two_sum(lo[k], two_sum(hi[k], p));
+                    ll[k] = __fadd_rn(ll[k], __fadd_rn(e, f));
                     mx[k] = fmaxf(mx[k], fabsf(q[k]));
                 }
             }
@@ -209,25 +219,35 @@ __global__ void __launch_bounds__(256) k_l21_norm_pairs(const float* __restrict_
         for (int k = 0; k < 2; ++k) {
             const float s = hi[k];
             const float wr = w_rows ? w_rows[(int64_t)b * N + pix + k] : 1.f;
-            if (s >= 0x1p-85f && s <= 0x1p126f) {
-                const float y = rsqrtf(s), h = 0.5f * y;
-                float r = s * y;
-                r = fmaf(h, fmaf(-r, r, s), r);
-                const float c = h * (__fmaf_rn(-r, r, s) + lo[k]);   // root = r + c
-                acc = fma((double)r + (double)c, (double)wr, acc);
-            } else if (mx[k] != 0.f || !(s == 0.f)) {
-                double d = 0.0;
-                for (int l = 0; l < L; ++l) {
-                    const double q = (double)row[(int64_t)l * N + k];
-                    d += q * q;
-                }
-                acc += sqrt(d) * (double)wr;
+            const float y = rsqrtf(s), h = 0.5f * y;
+            float r = s * y;
+            r = fmaf(h, fmaf(-r, r, s), r);
+            const float p = __fmul_rn(r, wr);
+            if (s >= 0x1p-85f && s <= 0x1p126f && fabsf(p) >= 0x1p-60f && fabsf(p) <= 0x1p120f) {
+                const float q = __fmul_rn(r, r);
+                float m = __fsub_rn(s, q);   // s - r^2 = m + rest (the difference is exact)
+                float rest = two_sum(m, -__fmaf_rn(r, r, -q));
+                rest = __fadd_rn(__fadd_rn(rest, two_sum(m, lo[k])), ll[k]);
+                const float c = h * m, z = __fmul_rn(2.f * r, c);
+                const float d = __fsub_rn(__fsub_rn(m, z), __fmaf_rn(2.f * r, c, -z));
+                const float c2 = h * (__fadd_rn(d, rest) - c * c);
+                const float cw = __fmul_rn(c, wr);
+                const float e = two_sum(slo, __fmaf_rn(r, wr, -p));
+                const float f = two_sum(slo, cw);
+                sll = __fadd_rn(sll, __fadd_rn(__fadd_rn(e, f), fmaf(c2, wr, __fmaf_rn(c, wr, -cw))));
+                acc += (double)p;
             } else {
-                acc += 0.0 * (double)wr;   // a zero row (NaN for a non-finite weight)
+                double d = 0.0;
+                if (mx[k] != 0.f || !(s == 0.f))   // not a zero row
+                    for (int l = 0; l < L; ++l) {
+                        const double t = (double)row[(int64_t)l * N + k];
+                        d = fma(t, t, d);
+                    }
+                acc += sqrt(d) * (double)wr;
             }
         }
     }
-    acc = block_sum(acc, red);
+    acc = block_sum(acc + ((double)slo + (double)sll), red);
     if (threadIdx.x == 0) part[blockIdx.x] = acc;
 }
 
@@ -329,8 +349,8 @@ hs_status l21_norm(Plan* p, const void* A, const void* w_rows, double* out_dev, 
     const int64_t N = p->N();
     int nb = 512;
     if (p->prec == HS_F32 && N % 2 == 0 && (uintptr_t)A % 8 == 0) {
-        nb = (int)std::min<int64_t>(nblk(NB * (N / 2), 256), 152 * 6);
-        k_l21_norm_pairs<<<nb, 256, 0, s>>>((const float*)A, (const float*)w_rows, p->g.L, N, p->part);
+        nb = (int)std::min<int64_t>(nblk(NB * (N / 2), 256), 152 * 5);   // 48 registers: 5 CTAs to an SM
+        k_l21_norm_exact<<<nb, 256, 0, s>>>((const float*)A, (const float*)w_rows, p->g.L, N, p->part);
     } else if (p->prec == HS_F32)
         k_l21_norm<float><<<nb, 256, 0, s>>>((const float*)A, (const float*)w_rows, p->g.L, N, p->part);
     else
