@@ -537,6 +537,18 @@ __global__ void __launch_bounds__(EIG_COLD_T, 1) k_eig_cold(const double* __rest
         emax = 0;
     }
     __syncthreads();
+    // The sweeps run on S times a power of two that brings its largest diagonal entry to [1, 2):
+    // the sum of all its squares, which decides whether to sweep, left the FP32 range from singular
+    // values of 1e9 on (and the sweeps were left out). In range no bit depends on it.
+    // (The largest exponent from the high words; scaled in FP32 while that cannot overflow: FP64 multiply-adds
+    // and the library's scalbn took 4 us here.)
+    int mh = 0;
+    for (int k = tid & 31; k < L; k += 32) mh = max(mh, __double2hiint(Sd[k * LDD + k]));
+    mh = __reduce_max_sync(0xffffffffu, mh) >> 20;
+    const int ex = mh > 0 && mh < 2047 ? mh - 1023 : 0;
+    const bool near = abs(ex) <= 64;
+    const double down = __hiloint2double((1023 - ex) << 20, 0), up = __hiloint2double((1023 + ex) << 20, 0);
+    const float downf = (float)down;
     // ---- 1. FP32 Jacobi, position k = indices 4k .. 4k + 3 at the start of every sweep.
     // Threads of the lower half hold blocks of A, those of the upper half blocks of V and apply a
     // round's rotations while the next round's are computed.
@@ -550,7 +562,8 @@ __global__ void __launch_bounds__(EIG_COLD_T, 1) k_eig_cold(const double* __rest
         for (int q = 0; q < 4; ++q) {
             const int i = 4 * I + p, j = 4 * J + q;
             if (half) a[p][q] = (in && i == j) ? 1.f : 0.f;
-            else a[p][q] = (in && i < L && j < L) ? (float)Sd[i * LDD + j] : 0.f;
+            else if (!in || i >= L || j >= L) a[p][q] = 0.f;
+            else a[p][q] = near ? (float)Sd[i * LDD + j] * downf : (float)(Sd[i * LDD + j] * down);
         }
     constexpr int PA[6] = {0, 1, 0, 1, 0, 2}, PB[6] = {2, 3, 3, 2, 1, 3};
     // blocks advance: first block of position 0 stays, position 1 gets position 0's second,
@@ -721,10 +734,10 @@ __global__ void __launch_bounds__(EIG_COLD_T, 1) k_eig_cold(const double* __rest
             const float lj = isnan(lamf[j]) ? -INFINITY : lamf[j];
             rk += (lj > li) || (lj == li && j < tid);
         }
-        lam32[tid] = (double)lamf[tid];
+        lam32[tid] = (double)lamf[tid] * up;
         order[rk] = tid;
         const double c = thr * (w_sv ? w_sv[rk] : 1.0) * (1.0 - 1e-3);
-        if ((double)fmaxf(li, 0.f) > c * c) atomicMax(&r_act, rk + 1);
+        if ((double)fmaxf(li, 0.f) * up > c * c) atomicMax(&r_act, rk + 1);
     }
     __syncthreads();
     const int r = r_act;
