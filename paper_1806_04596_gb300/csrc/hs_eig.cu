@@ -65,9 +65,13 @@ __device__ __forceinline__ void jac_rot(float app, float aqq, float apq, float& 
     s = t * c;
 }
 // FP64: the division and the roots of the library cost ~20 dependent FP64 instructions
-// each at 1/64 of the FP32 rate, and a round waits for them. The tangent is taken to
-// FP32 accuracy (a rotation then leaves ~1e-7 of a_pq, which later rounds remove);
-// what has to be FP64 is c^2 + s^2 = 1: c = (1 + t^2)^-1/2 by two Newton steps.
+// each at 1/64 of the FP32 rate, and a round waits for them. The tangent is taken from the
+// approximate FP64 reciprocal (about 20 bits) and FP32: a rotation then leaves ~1e-6 of a_pq, which
+// later rounds remove. What has to be FP64 is c^2 + s^2 = 1: one Newton step of (1 + t^2)^-1/2,
+// then c and s both by the first order of what 1 - c^2 - s^2 (exact to 2^-106 by fused
+// multiply-adds) still is. With a second Newton step in its place the rounding of c alone, always the same
+// way, stretched the 64 columns of V by 8e-15 in nine sweeps (now 2e-16; the prox of a
+// 60-channel cube with 3 active pairs was 1.2e-14 off for it).
 __device__ __forceinline__ void jac_rot(double app, double aqq, double apq, double& c, double& s) {
     double r;
     asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(2.0 * apq));
@@ -77,9 +81,11 @@ __device__ __forceinline__ void jac_rot(double app, double aqq, double apq, doub
     const double u = fma(t, t, 1.0);
     double y = (double)rsqrtf((float)u);
     y = fma(0.5 * y, fma(-(u * y), y, 1.0), y);
-    y = fma(0.5 * y, fma(-(u * y), y, 1.0), y);
     c = y;
     s = t * y;
+    const double e = 0.5 * fma(-s, s, fma(-c, c, 1.0));
+    c = fma(e, c, c);
+    s = fma(e, s, s);
 }
 
 // Cyclic Jacobi, round-robin parallel ordering, on the symmetric N x N matrix
