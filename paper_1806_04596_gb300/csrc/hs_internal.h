@@ -106,6 +106,7 @@ struct Plan {
     bool half = true;
     std::vector<float> uv_h;           // uv of FP32 plans the nuclear prior can use (plane_plan)
     std::weak_ptr<Plan> plane;         // whole-plane layout shared by the states that use it
+    std::shared_ptr<Plan> plane_keep;  // the same, kept for later states (null under a device limit)
     std::mutex plane_mu;
     int levels = 4;
     int J = 8, o = 2;
@@ -214,6 +215,7 @@ hs_status lib_alloc(void** ptr, size_t bytes);
 void lib_free(void* ptr, size_t bytes);
 void set_device_limit(int64_t bytes);
 int64_t device_bytes_held();
+int64_t device_limit();   // 0: none
 
 // ---------------------------------------------------------------- host tables
 hs_status daubechies_lowpass(int p, double* out);

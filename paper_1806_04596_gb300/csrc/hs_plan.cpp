@@ -47,6 +47,7 @@ static std::atomic<int64_t> g_lib_limit{0};
 
 void set_device_limit(int64_t bytes) { g_lib_limit.store(bytes < 0 ? 0 : bytes); }
 int64_t device_bytes_held() { return g_lib_bytes.load(); }
+int64_t device_limit() { return g_lib_limit.load(); }
 
 hs_status lib_alloc(void** ptr, size_t bytes) {
     *ptr = nullptr;
@@ -505,6 +506,43 @@ static hs_status autotune(Plan* p, cudaStream_t s) {
     return HS_OK;
 }
 
+// Tables that depend on the grid alone: kernel pieces, Z scale, twiddles, channel offsets.
+static hs_status build_tables(Plan* p) {
+    const Geo& g = p->g;
+    const int Kx = g.Kx, Ky = g.Ky;
+    HS_TRY(upload(p, (void**)&p->off_d, p->off_h));
+    std::vector<double> kbc;
+    p->kb_terms = p->prec == HS_F32 ? KB_TERMS_F32 : KB_TERMS_F64;
+    p->kb_fit_err = kb_poly_fit(p->J, p->beta, p->kb_terms, &kbc);
+    p->kbc_h = kbc;
+    std::vector<double> cx(g.nx), cy(g.ny);
+    for (int i = 0; i < g.nx; ++i) cx[i] = 1.0 / kb_phihat((double)(i - g.nx / 2) / Kx, p->J, p->beta);
+    for (int i = 0; i < g.ny; ++i) cy[i] = 1.0 / kb_phihat((double)(i - g.ny / 2) / Ky, p->J, p->beta);
+    std::vector<double> twx(2 * (size_t)Kx), twy(2 * (size_t)Ky);
+    for (int m = 0; m < Kx; ++m) {
+        twx[2 * m] = std::cos(2.0 * M_PI * m / Kx);
+        twx[2 * m + 1] = -std::sin(2.0 * M_PI * m / Kx);
+    }
+    for (int m = 0; m < Ky; ++m) {
+        twy[2 * m] = std::cos(2.0 * M_PI * m / Ky);
+        twy[2 * m + 1] = -std::sin(2.0 * M_PI * m / Ky);
+    }
+    if (p->prec == HS_F32) {
+        HS_TRY(upload_real<float>(p, &p->kbc, kbc));
+        HS_TRY(upload_real<float>(p, &p->cxs, cx));
+        HS_TRY(upload_real<float>(p, &p->cys, cy));
+        HS_TRY(upload_real<float>(p, &p->twx, twx));
+        HS_TRY(upload_real<float>(p, &p->twy, twy));
+    } else {
+        HS_TRY(upload_real<double>(p, &p->kbc, kbc));
+        HS_TRY(upload_real<double>(p, &p->cxs, cx));
+        HS_TRY(upload_real<double>(p, &p->cys, cy));
+        HS_TRY(upload_real<double>(p, &p->twx, twx));
+        HS_TRY(upload_real<double>(p, &p->twy, twy));
+    }
+    return HS_OK;
+}
+
 // Everything of a plan that depends on the coverage and on the plane kept (half
 // or whole): sorted order, coordinates, work lists, tables, grid scratch.
 // uvh, wh, uh: caller order (wh, uh empty for 1).
@@ -829,40 +867,8 @@ static hs_status build_layout(Plan* p, const std::vector<double>& uvh, const std
         }
     }
     if (sweep && !(p->flags & HS_PLAN_COMPENSATED)) p->n_ent = p->n_sw_ent;
-    HS_TRY(upload(p, (void**)&p->off_d, p->off_h));
-
-    // tables
-    std::vector<double> kbc;
-    p->kb_terms = p->prec == HS_F32 ? KB_TERMS_F32 : KB_TERMS_F64;
-    p->kb_fit_err = kb_poly_fit(p->J, p->beta, p->kb_terms, &kbc);
-    p->kbc_h = kbc;
-    std::vector<double> cx(g.nx), cy(g.ny);
-    for (int i = 0; i < g.nx; ++i) cx[i] = 1.0 / kb_phihat((double)(i - g.nx / 2) / Kx, p->J, p->beta);
-    for (int i = 0; i < g.ny; ++i) cy[i] = 1.0 / kb_phihat((double)(i - g.ny / 2) / Ky, p->J, p->beta);
-    std::vector<double> twx(2 * (size_t)Kx), twy(2 * (size_t)Ky);
-    for (int m = 0; m < Kx; ++m) {
-        twx[2 * m] = std::cos(2.0 * M_PI * m / Kx);
-        twx[2 * m + 1] = -std::sin(2.0 * M_PI * m / Kx);
-    }
-    for (int m = 0; m < Ky; ++m) {
-        twy[2 * m] = std::cos(2.0 * M_PI * m / Ky);
-        twy[2 * m + 1] = -std::sin(2.0 * M_PI * m / Ky);
-    }
-    if (p->prec == HS_F32) {
-        HS_TRY(upload_real<float>(p, &p->kbc, kbc));
-        HS_TRY(upload_real<float>(p, &p->cxs, cx));
-        HS_TRY(upload_real<float>(p, &p->cys, cy));
-        HS_TRY(upload_real<float>(p, &p->twx, twx));
-        HS_TRY(upload_real<float>(p, &p->twy, twy));
-    } else {
-        HS_TRY(upload_real<double>(p, &p->kbc, kbc));
-        HS_TRY(upload_real<double>(p, &p->cxs, cx));
-        HS_TRY(upload_real<double>(p, &p->cys, cy));
-        HS_TRY(upload_real<double>(p, &p->twx, twx));
-        HS_TRY(upload_real<double>(p, &p->twy, twy));
-    }
-
-    if (p->half) {   // the whole-plane layout of the same plan uses this scratch too (plane_plan)
+    if (p->half) {   // the whole-plane layout of the same plan uses these tables and this scratch (plane_plan)
+        HS_TRY(build_tables(p));
         const bool wide = p->prec == HS_F32 && L <= MAX_L_NUC;
         HS_TRY(plan_alloc(p, &p->grid, (size_t)L * Ky * (wide ? Kx : g.Kw) * p->csize()));
         HS_TRY(plan_alloc(p, &p->tmp, (size_t)L * g.ny * (wide ? Kx : g.Kc) * p->csize()));
@@ -1021,9 +1027,11 @@ hs_status plan_create(Plan** out, int nx, int ny, int L, const int64_t* vis_offs
 }
 
 // The whole-plane companion of an FP32 plan: same coverage, blocks, weights and
-// flags, lists and coordinates of its own, the plan's grid scratch (as the plan's own calls
-// and every state on it use that, in stream order); p stays unchanged but for the
-// shared reference.
+// flags, lists and coordinates of its own, the plan's tables and grid scratch (as the plan's own
+// calls and every state on it use that, in stream order); p stays unchanged but for the
+// shared reference. The plan keeps it for its next states (building it again took 38 ms per
+// state at 256 x 256, L = 60, where the state itself takes 0.7), but under a device limit
+// it goes with the last state that uses it.
 static hs_status make_plane(Plan* p, std::shared_ptr<Plan>* out, cudaStream_t s);
 hs_status plane_plan(Plan* p, std::shared_ptr<Plan>* out, cudaStream_t s) {
     return no_throw([&]() { return make_plane(p, out, s); });
@@ -1053,6 +1061,15 @@ static hs_status make_plane(Plan* p, std::shared_ptr<Plan>* out, cudaStream_t s)
     c->blk_off_h = p->blk_off_h;
     c->blk_ch = p->blk_ch;
     c->nblk = p->nblk;
+    c->off_d = p->off_d;   // tables of the plan (a state never outlives it)
+    c->kb_terms = p->kb_terms;
+    c->kb_fit_err = p->kb_fit_err;
+    c->kbc_h = p->kbc_h;
+    c->kbc = p->kbc;
+    c->cxs = p->cxs;
+    c->cys = p->cys;
+    c->twx = p->twx;
+    c->twy = p->twy;
     const int64_t M = p->M_total;
     std::vector<double> uvh(p->uv_h.begin(), p->uv_h.end()), wh, uh;
     if (p->w_sorted || p->u_sorted) {   // back to caller order
@@ -1101,6 +1118,7 @@ static hs_status make_plane(Plan* p, std::shared_ptr<Plan>* out, cudaStream_t s)
     c->k0y_h.shrink_to_fit();
     HS_CHECK_CUDA(cudaStreamSynchronize(s));
     p->plane = c;
+    if (!device_limit()) p->plane_keep = c;
     *out = c;
     return HS_OK;
 }
