@@ -882,6 +882,22 @@ static hs_status build_layout(Plan* p, const std::vector<double>& uvh, const std
     return HS_OK;
 }
 
+// Room for the tap tables of an FP64 plan (128 bytes per visibility, up to TAPS_MAX). They are
+// taken from memory nobody asked for: under a device limit only where the half plane saves as
+// much of the grid scratch, so that a plan never takes the room of the states and plans that
+// fit beside one with the whole plane and no tables; without a limit while half of the device's memory
+// stays free.
+static bool taps_fit(const Plan* p) {
+    const Geo& g = p->g;
+    const int64_t need = 16 * 8 * p->M_total;
+    if (need > TAPS_MAX) return false;
+    const int64_t saved = (int64_t)g.L * ((int64_t)g.Ky * (g.Kx - g.Kw) + (int64_t)g.ny * (g.Kx - g.Kc)) * (int64_t)p->csize() -
+                          (int64_t)(g.L * sizeof(int4));
+    if (need <= saved) return true;
+    size_t avail = 0, total = 0;
+    return device_limit() == 0 && cudaMemGetInfo(&avail, &total) == cudaSuccess && avail >= total / 2 + (size_t)need;
+}
+
 static hs_status build(Plan* p, const int64_t* vis_offsets, int nblocks, const int64_t* block_offsets,
                        const void* uv, const void* weights, const void* precond, cudaStream_t s) {
     Geo& g = p->g;
@@ -954,7 +970,7 @@ static hs_status build(Plan* p, const int64_t* vis_offsets, int nblocks, const i
     HS_TRY(plan_alloc(p, (void**)&p->dscal, sizeof(double) * 6 * std::max(L, 1)));
     HS_TRY(plan_alloc(p, (void**)&p->err_d, sizeof(int)));
     HS_CHECK_CUDA(cudaMemsetAsync(p->err_d, 0, sizeof(int), s));
-    if (p->prec == HS_F64 && M > 0 && 16 * 8 * M <= TAPS_MAX) {   // optional: without room the taps are evaluated
+    if (p->prec == HS_F64 && M > 0 && taps_fit(p)) {   // optional: else the taps are evaluated
         if (plan_alloc(p, &p->taps, (size_t)M * 16 * sizeof(double)) == HS_OK) HS_TRY(nufft_taps(p, s));
         else clear_error();
     }
