@@ -586,8 +586,9 @@ __global__ void k_gather_z2(const double2* __restrict__ in, const int* __restric
         out[i] = gather_one(in, perm[i]);
 }
 
-hs_status hs_pd_state_create(hs_plan_t plan, const void* Y, const double* eps,
-                             const hs_pd_params* prm, hs_pd_state_t* out, void* stream) {
+// whole: the data term on the whole-plane layout (plane_plan).
+static hs_status state_create(hs_plan_t plan, const void* Y, const double* eps, const hs_pd_params* prm, bool whole,
+                              hs_pd_state_t* out, void* stream) {
     clear_error();
     CHECK_PLAN(plan);
     if (out == nullptr || prm == nullptr || eps == nullptr || (Y == nullptr && plan->p->M_total > 0))
@@ -611,7 +612,7 @@ hs_status hs_pd_state_create(hs_plan_t plan, const void* Y, const double* eps,
     const int64_t M = p->M_total;
     hs_status e = HS_OK;
     st->dp = p;
-    if (prm->use_nuclear && p->prec == HS_F32 && M > 0) {
+    if (whole && prm->use_nuclear && p->prec == HS_F32 && M > 0) {
         HS_TRY(plane_plan(p, &st->plane, s));
         st->dp = st->plane.get();
     }
@@ -699,6 +700,15 @@ hs_status hs_pd_state_create(hs_plan_t plan, const void* Y, const double* eps,
     HS_TRY(cu(cudaStreamSynchronize(s), "sync"));
     *out = st.release();
     return HS_OK;
+}
+
+hs_status hs_pd_state_create(hs_plan_t plan, const void* Y, const double* eps,
+                             const hs_pd_params* prm, hs_pd_state_t* out, void* stream) {
+    const hs_status st = state_create(plan, Y, eps, prm, true, out, stream);
+    if (st != HS_ERR_NOMEM || plan == nullptr || plan->p == nullptr || plan->p->prec != HS_F32) return st;
+    // no room for the whole-plane layout beside the state: iterate on the plan's own half plane
+    drop_plane(plan->p);
+    return state_create(plan, Y, eps, prm, false, out, stream);
 }
 
 hs_status hs_pd_set_data(hs_pd_state_t st, const void* Y, const double* eps, void* stream) {

@@ -160,8 +160,8 @@ struct Plan {
     void* grid = nullptr;              // L * Ky * Kw complex
     void* tmp = nullptr;               // L * ny * Kc complex
     void* vis = nullptr;               // M_total complex (sorted order)
-    void* dwt_a = nullptr;             // 8 * L * N reals
-    void* dwt_b = nullptr;             // 8 * L * N reals
+    void* dwt_a = nullptr;             // 8 * L * N / 4 reals
+    void* dwt_b = nullptr;             // 8 * L * N / 4 reals
     double* part = nullptr;            // partial sums (size part_n doubles)
     int64_t part_n = 0;
     double* gram = nullptr;            // MAX_L_NUC^2 doubles
@@ -201,6 +201,7 @@ struct Plan {
 // L = 60: 5e-6 .. 1.8e-4 between the two Gram forms), so those solves keep the
 // whole-plane summation orders and reproduce their earlier iterates bit for bit.
 hs_status plane_plan(Plan* p, std::shared_ptr<Plan>* out, cudaStream_t s);
+void drop_plane(Plan* p);   // the plan's own reference to it
 // FFT of the whole plane (hs_fft_plane.cu; FP32).
 hs_status plane_fft_forward(Plan* p, const void* X, cudaStream_t s);
 hs_status plane_fft_cols_inv(Plan* p, const void* grid, void* tmp, int l0, int nl, cudaStream_t s);

@@ -956,8 +956,9 @@ static hs_status build(Plan* p, const int64_t* vis_offsets, int nblocks, const i
     // scratch
     const size_t rs = p->rsize(), cs = p->csize();
     const int64_t N = p->N();
-    HS_TRY(plan_alloc(p, &p->dwt_a, (size_t)NW * L * N * rs));
-    HS_TRY(plan_alloc(p, &p->dwt_b, (size_t)NW * L * N * rs));
+    // lowpass blocks between wavelet levels: the finest a level reads or writes is N / 4
+    HS_TRY(plan_alloc(p, &p->dwt_a, (size_t)NW * L * (N / 4) * rs));
+    HS_TRY(plan_alloc(p, &p->dwt_b, (size_t)NW * L * (N / 4) * rs));
     HS_TRY(plan_alloc(p, &p->xbuf, (size_t)L * N * rs));
     HS_TRY(plan_alloc(p, &p->xbuf2, (size_t)L * N * rs));
     const int64_t nbx = (Mmax + DEGRID_CHUNK - 1) / DEGRID_CHUNK;
@@ -1051,6 +1052,11 @@ hs_status plan_create(Plan** out, int nx, int ny, int L, const int64_t* vis_offs
 static hs_status make_plane(Plan* p, std::shared_ptr<Plan>* out, cudaStream_t s);
 hs_status plane_plan(Plan* p, std::shared_ptr<Plan>* out, cudaStream_t s) {
     return no_throw([&]() { return make_plane(p, out, s); });
+}
+
+void drop_plane(Plan* p) {
+    std::lock_guard<std::mutex> lock(p->plane_mu);
+    p->plane_keep.reset();
 }
 
 static hs_status make_plane(Plan* p, std::shared_ptr<Plan>* out, cudaStream_t s) {

@@ -54,3 +54,60 @@ def test_fp64_tables_leave_the_states_room(hs, M):
         assert rel(host(plan.phi_fwd(dev(c["X"], "f64"))), oracle_op(c).forward(c["X"])) <= TOL["f64"]
     finally:
         hs.set_device_limit(0)
+
+
+@pytest.mark.parametrize("M", [(2000, 1503, 0, 911), (60000, 40000, 50000, 0)])
+def test_fp32_states_fit_beside_one_set_of_lists(hs, M):
+    """A state with the nuclear prior where the limit leaves room for the state alone: it
+    iterates without a second layout, to the iterates of a state that has one (FP32 sums
+    in another order: 1e-5 an operator, which the warm-started eigensolver turns into at most
+    4e-4 of the image in ten iterations; three here)."""
+    c = ragged_case(n=64, L=4, M=M, seed=22)
+    plan = make_plan(c, "f32")
+    free = _state(hs, plan, c)
+    free.solve(3, graph=False)
+    want = host(free.get()[0])
+    del free, plan
+    plan = make_plan(c, "f32")
+    jas = _state(hs, plan, c, use_nuclear=False)
+    before = hs.device_bytes()
+    jas2 = _state(hs, plan, c, use_nuclear=False)
+    one = hs.device_bytes() - before
+    del jas, jas2
+    before = hs.device_bytes()
+    try:
+        hs.set_device_limit(before + one)
+        st = _state(hs, plan, c)
+        assert hs.device_bytes() <= before + one
+        st.solve(3, graph=True)
+        assert rel(host(st.get()[0]), want) <= 1e-4
+        hs.set_device_limit(before + one - 4096)
+        with pytest.raises(hs.HSError) as e:
+            _state(hs, plan, c)
+        assert e.value.status == hs.HS_ERR_NOMEM
+        assert hs.device_bytes() == before + one       # nothing left of the attempt
+    finally:
+        hs.set_device_limit(0)
+
+
+@pytest.mark.parametrize("prec", ["f32", "f64"])
+def test_plan_and_state_hold_no_more_than_with_one_layout(hs, prec):
+    """At a visibility and a half per pixel and channel, the bytes of a plan with the whole
+    plane's grid, one set of lists (24 bytes a visibility, 40 in FP64) and wavelet scratch of two
+    coefficient cubes."""
+    n, L = 128, 8
+    m = 3 * n * n // 2
+    c = ragged_case(n=n, L=L, M=(m,) * L, seed=23)
+    r = 4 if prec == "f32" else 8
+    K = 2 * n
+    before = hs.device_bytes()
+    try:
+        hs.set_device_limit(1 << 40)
+        plan = make_plan(c, prec)
+        st = _state(hs, plan, c)
+        N = n * n * L
+        whole = 2 * r * L * (K * K + n * K) + r * (16 + 2) * N + (2 * r + 8 + 4 * r) * m * L + (1 << 20)
+        assert hs.device_bytes() - before <= whole + _state_bytes(c, r)
+        del st
+    finally:
+        hs.set_device_limit(0)
