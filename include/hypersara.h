@@ -159,7 +159,7 @@ typedef struct {
     int kb_terms;                 /* coefficients per kernel polynomial piece */
     double kb_beta;
     double kb_fit_max_err;        /* max |poly - phi| / phi(0) of the kernel fit */
-    int64_t device_bytes;         /* device memory held by the plan */
+    int64_t device_bytes;         /* device memory held by the plan (with the second layout of its states) */
     int nblocks;                  /* data blocks (L unless created with hs_plan_create_blocks) */
     int gram_tc;                  /* FP32 Gram matrix on the tensor cores (1) or CUDA cores (0) */
     int sweep_hmax, sweep_cap;    /* sweep gridding: rows per work item, window cap per list */

@@ -217,7 +217,7 @@ hs_status hs_plan_info(hs_plan_t plan, hs_plan_info_t* info) {
     info->kb_terms = p->kb_terms;
     info->kb_beta = p->beta;
     info->kb_fit_max_err = p->kb_fit_err;
-    info->device_bytes = p->device_bytes;
+    info->device_bytes = p->device_bytes + plane_bytes(plan->p);
     info->nblocks = p->nblk;
     info->gram_tc = p->prec == HS_F32 ? p->gram_tc : 0;
     info->sweep_hmax = p->sweep_hmax;

@@ -202,6 +202,7 @@ struct Plan {
 // whole-plane summation orders and reproduce their earlier iterates bit for bit.
 hs_status plane_plan(Plan* p, std::shared_ptr<Plan>* out, cudaStream_t s);
 void drop_plane(Plan* p);   // the plan's own reference to it
+int64_t plane_bytes(Plan* p);   // device memory it holds (0 without one)
 // FFT of the whole plane (hs_fft_plane.cu; FP32).
 hs_status plane_fft_forward(Plan* p, const void* X, cudaStream_t s);
 hs_status plane_fft_cols_inv(Plan* p, const void* grid, void* tmp, int l0, int nl, cudaStream_t s);

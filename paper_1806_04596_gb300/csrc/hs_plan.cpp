@@ -1059,6 +1059,12 @@ void drop_plane(Plan* p) {
     p->plane_keep.reset();
 }
 
+int64_t plane_bytes(Plan* p) {
+    std::lock_guard<std::mutex> lock(p->plane_mu);
+    const std::shared_ptr<Plan> c = p->plane.lock();
+    return c ? c->device_bytes : 0;
+}
+
 static hs_status make_plane(Plan* p, std::shared_ptr<Plan>* out, cudaStream_t s) {
     std::lock_guard<std::mutex> lock(p->plane_mu);
     *out = p->plane.lock();
