@@ -24,7 +24,6 @@
 #include <map>
 #include <memory>
 #include <mutex>
-#include <system_error>
 #include <thread>
 #include <tuple>
 #include <vector>
@@ -180,8 +179,9 @@ static void parallel_for(int n, int64_t items, const std::function<void(int)>& f
     };
     std::vector<std::thread> ts;
     try {
+        ts.reserve(nt);
         for (int t = 1; t < nt; ++t) ts.emplace_back(work);
-    } catch (const std::system_error&) {   // no more threads: the ones there are do the work
+    } catch (const std::exception&) {   // no more threads, or no memory for one: the ones there are do the work
     }
     work();
     for (auto& t : ts) t.join();
