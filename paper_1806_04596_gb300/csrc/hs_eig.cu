@@ -476,8 +476,9 @@ __global__ void __launch_bounds__(EIG_T) k_eig_mixed(const double* __restrict__ 
 //  * The FP64 dot products of the correction steps are split over 8 lanes each when there are
 //    few: one thread per dot product left 60 dependent FP64 multiply-adds to wait for.
 //  * The last orthonormalisation is a product with the inverse Cholesky factor to first
-//    order (G = I + E: X (I - U), U = strict upper part of E plus half its diagonal) when
-//    E is below 1e-8, so that E^2 is below FP64 rounding; else the factorisation.
+//    order (G = I + E: X (I - U), U = strict upper part of E plus half its diagonal) while no entry
+//    of E^2 (r active vectors: at most r times the largest entry squared) passes FP64 rounding; else
+//    the factorisation.
 // us per prox at 64 x 64, before -> after: L = 60 with 2 active pairs 499 -> 349, all 60 active
 // 1357 -> 1246; L = 20 146 -> 99; L = 6 74 -> 49. A round takes ~2300 cycles, of
 // which the rotations' serial chain and the barriers are the larger part.
@@ -822,7 +823,8 @@ __global__ void __launch_bounds__(EIG_COLD_T, 1) k_eig_cold(const double* __rest
                      const int i = k / r, c = k - i * r;
                      if (i > c) return;
                      Tb[i * LDD + c] = v.x;
-                     if (!(fabs(v.x - (i == c ? 1.0 : 0.0)) <= 1e-8)) atomicMax(&emax, 1);
+                     const double e = v.x - (i == c ? 1.0 : 0.0);
+                     if (!(r * e * e <= 1e-16)) atomicMax(&emax, 1);
                  });
         if (emax == 0) {   // X (I - U)
             each_dot(L * r,
