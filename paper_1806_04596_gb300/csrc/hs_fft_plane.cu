@@ -34,12 +34,12 @@ namespace {
 
 enum FftMode { ROW_FWD = 0, COL_FWD = 1, COL_INV = 2, ROW_INV = 3 };
 
-template <typename R> struct FftArgs {
+struct FftArgs {
     const void* in;
     void* out;
-    const Cx<R>* tw;   // exp(-2 pi i m / K), m < K
-    const R* cxs;      // Z scale along x (nx)
-    const R* cys;      // Z scale along y (ny)
+    const float2* tw;   // exp(-2 pi i m / K), m < K
+    const float* cxs;      // Z scale along x (nx)
+    const float* cys;      // Z scale along y (ny)
     int K, G, n8, rlast, npass;
     int lgK, lgG;      // log2 K, log2 G
     int nx, ny, Kx, Ky;
@@ -49,8 +49,8 @@ template <typename R> struct FftArgs {
 
 // A line is a row (l, iy) of the row modes or a column (l, kx) of the column
 // modes; la = channel, lb = iy or kx.
-template <typename R, int MODE>
-__device__ __forceinline__ void line_of(const FftArgs<R>& a, int line, int& la, int& lb) {
+template <int MODE>
+__device__ __forceinline__ void line_of(const FftArgs& a, int line, int& la, int& lb) {
     if (MODE == COL_FWD || MODE == COL_INV) {
         la = line >> a.lgKx;
         lb = line & (a.Kx - 1);
@@ -60,54 +60,52 @@ __device__ __forceinline__ void line_of(const FftArgs<R>& a, int line, int& la, 
     }
 }
 
-template <typename R, int MODE>
-__device__ __forceinline__ Cx<R> fft_load(const FftArgs<R>& a, int la, int lb, int k) {
-    typedef Cx<R> CT;
+template <int MODE>
+__device__ __forceinline__ float2 fft_load(const FftArgs& a, int la, int lb, int k) {
     if (MODE == ROW_FWD) {   // Z: pad and scale
         const int h = a.nx >> 1;
         int ix;
         if (k < h) ix = k + h;
         else if (k >= a.Kx - h) ix = k - a.Kx + h;
-        else return cx<R>(0, 0);
-        const R* X = (const R*)a.in;
-        return cx<R>(a.cys[lb] * a.cxs[ix] * X[((int64_t)la * a.ny + lb) * a.nx + ix], (R)0);
+        else return cx<float>(0, 0);
+        const float* X = (const float*)a.in;
+        return cx<float>(a.cys[lb] * a.cxs[ix] * X[((int64_t)la * a.ny + lb) * a.nx + ix], (float)0);
     } else if (MODE == COL_FWD) {   // only the ny image rows are nonzero
         const int h = a.ny >> 1;
         int iy;
         if (k < h) iy = k + h;
         else if (k >= a.Ky - h) iy = k - a.Ky + h;
-        else return cx<R>(0, 0);
-        return ((const CT*)a.in)[((int64_t)la * a.ny + iy) * a.Kx + lb];
+        else return cx<float>(0, 0);
+        return ((const float2*)a.in)[((int64_t)la * a.ny + iy) * a.Kx + lb];
     } else if (MODE == COL_INV) {
-        if (!row_reached(a.rng[la], k)) return cx<R>(0, 0);
-        return ((const CT*)a.in)[((int64_t)la * a.Ky + k) * a.Kx + lb];
+        if (!row_reached(a.rng[la], k)) return cx<float>(0, 0);
+        return ((const float2*)a.in)[((int64_t)la * a.Ky + k) * a.Kx + lb];
     } else {   // ROW_INV
-        if (!col_reached(a.rng[la], k)) return cx<R>(0, 0);
-        return ((const CT*)a.in)[((int64_t)la * a.ny + lb) * a.Kx + k];
+        if (!col_reached(a.rng[la], k)) return cx<float>(0, 0);
+        return ((const float2*)a.in)[((int64_t)la * a.ny + lb) * a.Kx + k];
     }
 }
 
-template <typename R, int MODE>
-__device__ __forceinline__ void fft_store(const FftArgs<R>& a, int la, int lb, int k, Cx<R> v) {
-    typedef Cx<R> CT;
+template <int MODE>
+__device__ __forceinline__ void fft_store(const FftArgs& a, int la, int lb, int k, float2 v) {
     if (MODE == ROW_FWD) {
-        if (col_reached(a.rng[la], k)) ((CT*)a.out)[((int64_t)la * a.ny + lb) * a.Kx + k] = v;
+        if (col_reached(a.rng[la], k)) ((float2*)a.out)[((int64_t)la * a.ny + lb) * a.Kx + k] = v;
     } else if (MODE == COL_FWD) {
-        if (row_reached(a.rng[la], k)) ((CT*)a.out)[((int64_t)la * a.Ky + k) * a.Kx + lb] = v;
+        if (row_reached(a.rng[la], k)) ((float2*)a.out)[((int64_t)la * a.Ky + k) * a.Kx + lb] = v;
     } else if (MODE == COL_INV) {   // keep the ny image rows
         const int h = a.ny >> 1;
         int iy;
         if (k < h) iy = k + h;
         else if (k >= a.Ky - h) iy = k - a.Ky + h;
         else return;
-        ((CT*)a.out)[((int64_t)la * a.ny + iy) * a.Kx + lb] = v;
+        ((float2*)a.out)[((int64_t)la * a.ny + iy) * a.Kx + lb] = v;
     } else {   // ROW_INV: crop, scale, real part
         const int h = a.nx >> 1;
         int ix;
         if (k < h) ix = k + h;
         else if (k >= a.Kx - h) ix = k - a.Kx + h;
         else return;
-        ((R*)a.out)[((int64_t)la * a.ny + lb) * a.nx + ix] = a.cys[lb] * a.cxs[ix] * v.x;
+        ((float*)a.out)[((int64_t)la * a.ny + lb) * a.nx + ix] = a.cys[lb] * a.cxs[ix] * v.x;
     }
 }
 
@@ -116,10 +114,9 @@ __device__ __forceinline__ void fft_store(const FftArgs<R>& a, int la, int lb, i
 // registers; NREP > 1 lets long column lines come G = 4 to a CTA, so that
 // every 32-byte sector of a column load is used, within 512 threads).
 // LGK_ / LGG_ > 0 fix log2 K and log2 G at compile time (0: from the arguments).
-template <typename R, int DIR, int MODE, int RAD, int LGR, int LGK_, int LGG_, int NREP>
-__device__ __forceinline__ void fft_pass(const FftArgs<R>& a, Cx<R>* sm, int lgNs, bool first,
+template <int DIR, int MODE, int RAD, int LGR, int LGK_, int LGG_, int NREP>
+__device__ __forceinline__ void fft_pass(const FftArgs& a, float2* sm, int lgNs, bool first,
                                          bool last, int line0) {
-    typedef Cx<R> CT;
     constexpr bool COLS = (MODE == COL_FWD || MODE == COL_INV);
     constexpr int PER = 8 / RAD * NREP;
     const int lgK = LGK_ > 0 ? LGK_ : a.lgK;
@@ -129,7 +126,7 @@ __device__ __forceinline__ void fft_pass(const FftArgs<R>& a, Cx<R>* sm, int lgN
     const int lgnb = lgK - LGR;
     const int nb = 1 << lgnb;
     const int lgstep = lgK - lgNs - LGR;
-    CT v[8 * NREP];
+    float2 v[8 * NREP];
     int gs[PER], js[PER];
 #pragma unroll
     for (int i = 0; i < PER; ++i) {
@@ -139,11 +136,11 @@ __device__ __forceinline__ void fft_pass(const FftArgs<R>& a, Cx<R>* sm, int lgN
         gs[i] = g;
         js[i] = j;
         int la = 0, lb = 0;
-        if (first) line_of<R, MODE>(a, line0 + g, la, lb);
+        if (first) line_of<MODE>(a, line0 + g, la, lb);
 #pragma unroll
         for (int r = 0; r < RAD; ++r) {
             const int k = j + r * nb;
-            v[i * RAD + r] = first ? fft_load<R, MODE>(a, la, lb, k)
+            v[i * RAD + r] = first ? fft_load<MODE>(a, la, lb, k)
                                    : sm[COLS ? (k * G + g) : (g * K + k)];
         }
     }
@@ -152,11 +149,11 @@ __device__ __forceinline__ void fft_pass(const FftArgs<R>& a, Cx<R>* sm, int lgN
     for (int i = 0; i < PER; ++i) {
         const int j = js[i];
         const int kk = j & ((1 << lgNs) - 1);
-        CT* u = v + i * RAD;
+        float2* u = v + i * RAD;
         if (lgNs > 0) {   // the first pass has unit twiddles
             if (RAD == 8) {
                 // w^1, w^2, w^4 from the table, the others as products (one rounding each)
-                CT t[8];
+                float2 t[8];
                 t[1] = a.tw[kk << lgstep];
                 t[2] = a.tw[(2 * kk) << lgstep];
                 t[4] = a.tw[(4 * kk) << lgstep];
@@ -172,37 +169,38 @@ __device__ __forceinline__ void fft_pass(const FftArgs<R>& a, Cx<R>* sm, int lgN
             } else {
 #pragma unroll
                 for (int r = 1; r < RAD; ++r) {
-                    CT t = a.tw[(kk * r) << lgstep];
+                    float2 t = a.tw[(kk * r) << lgstep];
                     if (DIR > 0) t.y = -t.y;
                     u[r] = cmul(u[r], t);
                 }
             }
         }
         if (RAD == 8) {
-            dft8<R, DIR>(u);
+            dft8<float, DIR>(u);
         } else if (RAD == 4) {
             dft4<DIR>(u[0], u[1], u[2], u[3]);
         } else {
-            CT t0 = cadd(u[0], u[1]);
+            float2 t0 = cadd(u[0], u[1]);
             u[1] = csub(u[0], u[1]);
             u[0] = t0;
         }
         const int base = ((j >> lgNs) << (lgNs + LGR)) + kk;
         const int g = gs[i];
         int la = 0, lb = 0;
-        if (last) line_of<R, MODE>(a, line0 + g, la, lb);
+        if (last) line_of<MODE>(a, line0 + g, la, lb);
 #pragma unroll
         for (int r = 0; r < RAD; ++r) {
             const int k = base + (r << lgNs);
-            if (last) fft_store<R, MODE>(a, la, lb, k, u[r]);
+            if (last) fft_store<MODE>(a, la, lb, k, u[r]);
             else sm[COLS ? (k * G + g) : (g * K + k)] = u[r];
         }
     }
     __syncthreads();
 }
 
-// A column group (at most 8 columns from a multiple of their number) that no window reaches.
-template <typename R, int MODE> __device__ __forceinline__ bool unreached(const FftArgs<R>& a, int line0) {
+// A column group that no window reaches: the columns no window reaches are one range, so both ends tell
+// (groups are 1 to 16 columns).
+template <int MODE> __device__ __forceinline__ bool unreached(const FftArgs& a, int line0) {
     if (MODE != COL_FWD && MODE != COL_INV) return false;
     const int la = line0 / a.Kx, c = line0 - la * a.Kx;
     return !col_reached(a.rng[la], c) && !col_reached(a.rng[la], c + a.G - 1);
@@ -211,35 +209,35 @@ template <typename R, int MODE> __device__ __forceinline__ bool unreached(const 
 // DIR = -1: forward transform (exp(-2 pi i kn / K)); DIR = +1: unnormalised inverse.
 // LGK_ > 0: K = 2^LGK_ lines of G = 2^LGG_ per CTA fixed at compile time (the
 // pass schedule and every index computation fold to constants); 0: generic.
-template <typename R, int DIR, int MODE, int LGK_, int LGG_, int NREP = 1>
-__global__ void __launch_bounds__(512, NREP > 1 ? 1 : (sizeof(R) == 4 ? 3 : 2)) k_plane_fft(FftArgs<R> a) {
+template <int DIR, int MODE, int LGK_, int LGG_, int NREP = 1>
+__global__ void __launch_bounds__(512, NREP > 1 ? 1 : 3) k_plane_fft(FftArgs a) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    Cx<R>* sm = reinterpret_cast<Cx<R>*>(smem_raw);
+    float2* sm = reinterpret_cast<float2*>(smem_raw);
     if constexpr (LGK_ > 0) {
         constexpr int N8 = LGK_ / 3, REM = LGK_ % 3, NPASS = N8 + (REM ? 1 : 0);
         const int line0 = blockIdx.x << LGG_;
-        if (unreached<R, MODE>(a, line0)) return;
+        if (unreached<MODE>(a, line0)) return;
 #pragma unroll
         for (int pass = 0; pass < NPASS; ++pass) {
             const bool first = (pass == 0), last = (pass == NPASS - 1);
-            if (pass < N8) fft_pass<R, DIR, MODE, 8, 3, LGK_, LGG_, NREP>(a, sm, 3 * pass, first, last, line0);
-            else if (REM == 2) fft_pass<R, DIR, MODE, 4, 2, LGK_, LGG_, NREP>(a, sm, 3 * pass, first, last, line0);
-            else fft_pass<R, DIR, MODE, 2, 1, LGK_, LGG_, NREP>(a, sm, 3 * pass, first, last, line0);
+            if (pass < N8) fft_pass<DIR, MODE, 8, 3, LGK_, LGG_, NREP>(a, sm, 3 * pass, first, last, line0);
+            else if (REM == 2) fft_pass<DIR, MODE, 4, 2, LGK_, LGG_, NREP>(a, sm, 3 * pass, first, last, line0);
+            else fft_pass<DIR, MODE, 2, 1, LGK_, LGG_, NREP>(a, sm, 3 * pass, first, last, line0);
         }
     } else {
         const int line0 = blockIdx.x * a.G;
-        if (unreached<R, MODE>(a, line0)) return;
+        if (unreached<MODE>(a, line0)) return;
         int lgNs = 0;
         for (int pass = 0; pass < a.npass; ++pass) {
             const bool first = (pass == 0), last = (pass == a.npass - 1);
             if (pass < a.n8) {
-                fft_pass<R, DIR, MODE, 8, 3, 0, 0, 1>(a, sm, lgNs, first, last, line0);
+                fft_pass<DIR, MODE, 8, 3, 0, 0, 1>(a, sm, lgNs, first, last, line0);
                 lgNs += 3;
             } else if (a.rlast == 4) {
-                fft_pass<R, DIR, MODE, 4, 2, 0, 0, 1>(a, sm, lgNs, first, last, line0);
+                fft_pass<DIR, MODE, 4, 2, 0, 0, 1>(a, sm, lgNs, first, last, line0);
                 lgNs += 2;
             } else {
-                fft_pass<R, DIR, MODE, 2, 1, 0, 0, 1>(a, sm, lgNs, first, last, line0);
+                fft_pass<DIR, MODE, 2, 1, 0, 0, 1>(a, sm, lgNs, first, last, line0);
                 lgNs += 1;
             }
         }
@@ -271,25 +269,24 @@ __device__ __forceinline__ void line_of_any(int line, int Kx, int ny, int& la, i
 // q-point DFT and writes it to out[(j / Ns) Ns q + (j mod Ns) + u Ns] (u < q);
 // after all passes the lines are in natural order. Twiddles come from the
 // K-point table w^m = exp(-2 pi i m / K) (conjugated for DIR = +1).
-template <typename R, int DIR, int MODE>
-__global__ void __launch_bounds__(512) k_plane_fft_mr(FftArgs<R> a, MrPlan mp) {
-    typedef Cx<R> CT;
+template <int DIR, int MODE>
+__global__ void __launch_bounds__(512) k_plane_fft_mr(FftArgs a, MrPlan mp) {
     constexpr bool COLS = (MODE == COL_FWD || MODE == COL_INV);
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int K = a.K, G = a.G, GK = G * K;
-    CT* src = reinterpret_cast<CT*>(smem_raw);
-    CT* dst = src + GK;
+    float2* src = reinterpret_cast<float2*>(smem_raw);
+    float2* dst = src + GK;
     const int line0 = blockIdx.x * G, tid = threadIdx.x, nthr = blockDim.x;
-    if (unreached<R, MODE>(a, line0)) return;
+    if (unreached<MODE>(a, line0)) return;
     for (int e = tid; e < GK; e += nthr) {   // consecutive threads: consecutive columns / row elements
         const int g = COLS ? e % G : e / K, k = COLS ? e / G : e % K;
         int la, lb;
         line_of_any<MODE>(line0 + g, a.Kx, a.ny, la, lb);
-        src[g * K + k] = fft_load<R, MODE>(a, la, lb, k);
+        src[g * K + k] = fft_load<MODE>(a, la, lb, k);
     }
     __syncthreads();
     auto tw = [&](int m) {
-        CT t = a.tw[m];
+        float2 t = a.tw[m];
         if (DIR > 0) t.y = -t.y;
         return t;
     };
@@ -299,7 +296,7 @@ __global__ void __launch_bounds__(512) k_plane_fft_mr(FftArgs<R> a, MrPlan mp) {
         for (int e = tid; e < G * nb; e += nthr) {
             const int g = e / nb, j = e - g * nb;
             const int k = j % Ns;
-            CT x[5], y[5];
+            float2 x[5], y[5];
 #pragma unroll
             for (int t = 0; t < 5; ++t)
                 if (t < q) x[t] = src[g * K + j + t * nb];
@@ -312,7 +309,7 @@ __global__ void __launch_bounds__(512) k_plane_fft_mr(FftArgs<R> a, MrPlan mp) {
 #pragma unroll
             for (int u = 0; u < 5; ++u) {
                 if (u >= q) break;
-                CT acc = x[0];
+                float2 acc = x[0];
 #pragma unroll
                 for (int t = 1; t < 5; ++t)
                     if (t < q) acc = cadd(acc, cmul(x[t], tw(((u * t) % q) * step)));
@@ -324,7 +321,7 @@ __global__ void __launch_bounds__(512) k_plane_fft_mr(FftArgs<R> a, MrPlan mp) {
                 if (u < q) dst[g * K + base + u * Ns] = y[u];
         }
         __syncthreads();
-        CT* t = src;
+        float2* t = src;
         src = dst;
         dst = t;
         Ns *= q;
@@ -333,7 +330,7 @@ __global__ void __launch_bounds__(512) k_plane_fft_mr(FftArgs<R> a, MrPlan mp) {
         const int g = COLS ? e % G : e / K, k = COLS ? e / G : e % K;
         int la, lb;
         line_of_any<MODE>(line0 + g, a.Kx, a.ny, la, lb);
-        fft_store<R, MODE>(a, la, lb, k, src[g * K + k]);
+        fft_store<MODE>(a, la, lb, k, src[g * K + k]);
     }
 }
 
@@ -368,9 +365,9 @@ static void radix_plan(int K, int* n8, int* rlast, int* npass) {
 }
 
 // nl channels from l0, starting at in / out (a channel range of the plan's cube).
-template <typename R, int DIR, int MODE>
+template <int DIR, int MODE>
 static hs_status launch_fft(Plan* p, const void* in, void* out, int l0, int nl, cudaStream_t s) {
-    FftArgs<R> a;
+    FftArgs a;
     a.in = in;
     a.out = out;
     a.nx = p->g.nx;
@@ -378,26 +375,25 @@ static hs_status launch_fft(Plan* p, const void* in, void* out, int l0, int nl, 
     a.Kx = p->g.Kx;
     a.Ky = p->g.Ky;
     a.rng = p->rng + l0;
-    a.cxs = (const R*)p->cxs;
-    a.cys = (const R*)p->cys;
+    a.cxs = (const float*)p->cxs;
+    a.cys = (const float*)p->cys;
     constexpr bool cols = (MODE == COL_FWD || MODE == COL_INV);
     const int K = cols ? p->g.Ky : p->g.Kx;
     a.K = K;
-    a.tw = (const Cx<R>*)(cols ? p->twy : p->twx);
+    a.tw = (const float2*)(cols ? p->twy : p->twx);
     if (!is_pow2(K) || !is_pow2(cols ? p->g.Kx : p->g.ny)) {   // mixed radix, generic indexing
         MrPlan mp;
         if (!mr_plan(K, &mp)) return fail(HS_ERR_ARG, "FFT: line length %d is not r 2^m with r in {1, 3, 5}", K);
         int G = 1;
         if (cols) {   // whole 32-byte sectors per column load where shared memory allows
-            const int want = (int)(32 / sizeof(Cx<R>)) > 0 ? (int)(32 / sizeof(Cx<R>)) : 1;
-            G = std::max(1, want);
-            while (G > 1 && (p->g.Kx % G != 0 || (size_t)2 * G * K * sizeof(Cx<R>) > (size_t)200 * 1024)) G >>= 1;
+            G = (int)(32 / sizeof(float2));
+            while (G > 1 && (p->g.Kx % G != 0 || (size_t)2 * G * K * sizeof(float2) > (size_t)200 * 1024)) G >>= 1;
         }
         a.G = G;
         const int nlines = nl * (cols ? p->g.Kx : p->g.ny);
-        const size_t smem = (size_t)2 * G * K * sizeof(Cx<R>);
+        const size_t smem = (size_t)2 * G * K * sizeof(float2);
         if (smem > (size_t)200 * 1024) return fail(HS_ERR_ARG, "FFT: line length %d too long", K);
-        k_plane_fft_mr<R, DIR, MODE><<<nlines / G, 512, smem, s>>>(a, mp);
+        k_plane_fft_mr<DIR, MODE><<<nlines / G, 512, smem, s>>>(a, mp);
         HS_CHECK_LAUNCH();
         return HS_OK;
     }
@@ -413,12 +409,12 @@ static hs_status launch_fft(Plan* p, const void* in, void* out, int l0, int nl, 
     int G, nlines, nrep = 1;
     if (cols) {
         // 512 threads per CTA so two CTAs share an SM (one loads while the other computes);
-        // lines longer than 1024 come 4 to a CTA (2 for FP64 at 4096: shared memory) with
+        // lines longer than 1024 come 4 to a CTA with
         // several butterflies per thread, so column loads use whole 32-byte sectors
         G = 512 / (K / 8);
         if (G > 16) G = 16;
         if (K >= 2048) {
-            G = (sizeof(R) == 8 && K >= 4096) ? 2 : 4;
+            G = 4;
             nrep = G * K / 8 / 512;
         }
         if (G > p->g.Kx) G = p->g.Kx;
@@ -433,19 +429,19 @@ static hs_status launch_fft(Plan* p, const void* in, void* out, int l0, int nl, 
     a.G = G;
     a.lgG = lg2(G);
     const int threads = G * K / 8 / nrep;
-    const size_t smem = (size_t)G * K * sizeof(Cx<R>);
+    const size_t smem = (size_t)G * K * sizeof(float2);
     const int blocks = nlines / G;
     if (blocks == 0) return HS_OK;
     // compile-time sizes for the common grids (G as chosen above for these K)
 #define HS_FFT_CT(LK, LG) \
     if (a.lgK == LK && a.lgG == LG && nrep == 1) { \
-        k_plane_fft<R, DIR, MODE, LK, LG><<<blocks, threads, smem, s>>>(a); \
+        k_plane_fft<DIR, MODE, LK, LG><<<blocks, threads, smem, s>>>(a); \
         HS_CHECK_LAUNCH(); \
         return HS_OK; \
     }
 #define HS_FFT_CT_REP(LK, LG, NR) \
     if (a.lgK == LK && a.lgG == LG && nrep == NR) { \
-        k_plane_fft<R, DIR, MODE, LK, LG, NR><<<blocks, threads, smem, s>>>(a); \
+        k_plane_fft<DIR, MODE, LK, LG, NR><<<blocks, threads, smem, s>>>(a); \
         HS_CHECK_LAUNCH(); \
         return HS_OK; \
     }
@@ -453,11 +449,7 @@ static hs_status launch_fft(Plan* p, const void* in, void* out, int l0, int nl, 
         HS_FFT_CT(9, 3)
         HS_FFT_CT(10, 2)
         HS_FFT_CT_REP(11, 2, 2)
-        if constexpr (sizeof(R) == 4) {
-            HS_FFT_CT_REP(12, 2, 4)
-        } else {
-            HS_FFT_CT_REP(12, 1, 2)
-        }
+        HS_FFT_CT_REP(12, 2, 4)
     } else {
         HS_FFT_CT(9, 2)
         HS_FFT_CT(10, 1)
@@ -467,34 +459,30 @@ static hs_status launch_fft(Plan* p, const void* in, void* out, int l0, int nl, 
 #undef HS_FFT_CT
 #undef HS_FFT_CT_REP
     if (nrep != 1) return fail(HS_ERR_ARG, "FFT: no kernel for K = %d with %d lines per CTA", K, G);
-    k_plane_fft<R, DIR, MODE, 0, 0><<<blocks, threads, smem, s>>>(a);
+    k_plane_fft<DIR, MODE, 0, 0><<<blocks, threads, smem, s>>>(a);
     HS_CHECK_LAUNCH();
     return HS_OK;
 }
 
-template <typename R, int DIR, int MODE, int LK, int LG, int NR = 1> static hs_status fft_attr1() {
-    HS_CHECK_CUDA(cudaFuncSetAttribute(k_plane_fft<R, DIR, MODE, LK, LG, NR>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+template <int DIR, int MODE, int LK, int LG, int NR = 1> static hs_status fft_attr1() {
+    HS_CHECK_CUDA(cudaFuncSetAttribute(k_plane_fft<DIR, MODE, LK, LG, NR>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        200 * 1024));
     return HS_OK;
 }
 
-template <typename R, int DIR, int MODE> static hs_status fft_attr() {
+template <int DIR, int MODE> static hs_status fft_attr() {
     constexpr bool cols = (MODE == COL_FWD || MODE == COL_INV);
-    HS_CHECK_CUDA(cudaFuncSetAttribute(k_plane_fft_mr<R, DIR, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    HS_CHECK_CUDA(cudaFuncSetAttribute(k_plane_fft_mr<DIR, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        200 * 1024));
-    HS_TRY((fft_attr1<R, DIR, MODE, 0, 0>()));
-    HS_TRY((fft_attr1<R, DIR, MODE, 9, cols ? 3 : 2>()));
-    HS_TRY((fft_attr1<R, DIR, MODE, 10, cols ? 2 : 1>()));
+    HS_TRY((fft_attr1<DIR, MODE, 0, 0>()));
+    HS_TRY((fft_attr1<DIR, MODE, 9, cols ? 3 : 2>()));
+    HS_TRY((fft_attr1<DIR, MODE, 10, cols ? 2 : 1>()));
     if constexpr (cols) {
-        HS_TRY((fft_attr1<R, DIR, MODE, 11, 2, 2>()));
-        if constexpr (sizeof(R) == 4) {
-            HS_TRY((fft_attr1<R, DIR, MODE, 12, 2, 4>()));
-        } else {
-            HS_TRY((fft_attr1<R, DIR, MODE, 12, 1, 2>()));
-        }
+        HS_TRY((fft_attr1<DIR, MODE, 11, 2, 2>()));
+        HS_TRY((fft_attr1<DIR, MODE, 12, 2, 4>()));
     } else {
-        HS_TRY((fft_attr1<R, DIR, MODE, 11, 0>()));
-        HS_TRY((fft_attr1<R, DIR, MODE, 12, 0>()));
+        HS_TRY((fft_attr1<DIR, MODE, 11, 0>()));
+        HS_TRY((fft_attr1<DIR, MODE, 12, 0>()));
     }
     return HS_OK;
 }
@@ -504,23 +492,23 @@ template <typename R, int DIR, int MODE> static hs_status fft_attr() {
 // Opt the kernels into large dynamic shared memory (when a whole-plane layout is
 // built, outside any stream capture).
 hs_status plane_fft_init() {
-    HS_TRY((fft_attr<float, -1, ROW_FWD>()));
-    HS_TRY((fft_attr<float, -1, COL_FWD>()));
-    HS_TRY((fft_attr<float, 1, COL_INV>()));
-    return fft_attr<float, 1, ROW_INV>();
+    HS_TRY((fft_attr<-1, ROW_FWD>()));
+    HS_TRY((fft_attr<-1, COL_FWD>()));
+    HS_TRY((fft_attr<1, COL_INV>()));
+    return fft_attr<1, ROW_INV>();
 }
 
 hs_status plane_fft_forward(Plan* p, const void* X, cudaStream_t s) {
-    HS_TRY((launch_fft<float, -1, ROW_FWD>(p, X, p->tmp, 0, p->g.L, s)));
-    return launch_fft<float, -1, COL_FWD>(p, p->tmp, p->grid, 0, p->g.L, s);
+    HS_TRY((launch_fft<-1, ROW_FWD>(p, X, p->tmp, 0, p->g.L, s)));
+    return launch_fft<-1, COL_FWD>(p, p->tmp, p->grid, 0, p->g.L, s);
 }
 
 hs_status plane_fft_cols_inv(Plan* p, const void* grid, void* tmp, int l0, int nl, cudaStream_t s) {
-    return launch_fft<float, 1, COL_INV>(p, grid, tmp, l0, nl, s);
+    return launch_fft<1, COL_INV>(p, grid, tmp, l0, nl, s);
 }
 
 hs_status plane_fft_rows_inv(Plan* p, const void* tmp, void* X, int l0, int nl, cudaStream_t s) {
-    return launch_fft<float, 1, ROW_INV>(p, tmp, X, l0, nl, s);
+    return launch_fft<1, ROW_INV>(p, tmp, X, l0, nl, s);
 }
 
 }  // namespace hs

@@ -155,7 +155,7 @@ struct Plan {
     void* twy = nullptr;               // Ky complex
     void* filt = nullptr;              // 8 * 2 * MAXF reals: lowpass, highpass per db_p
     // scratch
-    int4* rng = nullptr;               // per channel: the cells its windows reach (Reach below)
+    int4* rng = nullptr;               // per channel: the cells its windows reach (col_reached, row_reached)
     std::vector<int4> rng_h;           // the same on the host
     void* grid = nullptr;              // L * Ky * Kw complex
     void* tmp = nullptr;               // L * ny * Kc complex

@@ -511,17 +511,16 @@ __device__ __forceinline__ void ld4(const double* p, double* v) {
 // Partial Gram matrices S_ij = sum_n z_in z_jn, z = X (+ Xa), for L <= 64:
 // thread (bi, bj) of a 16 x 16 grid owns the 4 x 4 block of rows 4 bi .. 4 bi + 3
 // and columns 4 bj .. 4 bj + 3 (register blocking: per pixel two 4-wide shared
-// loads feed 16 FMAs). Runs of 32 pixels are summed in R and added into a
+// loads feed 16 FMAs). Runs of 32 pixels are summed in FP32 and added into a
 // (hi, lo) pair with the error-free two-sum (Knuth), so the accumulation across
 // runs is as exact as in FP64 without FP64 arithmetic; each CTA writes its
 // upper-triangle partials in FP64.
-template <typename R>
-__global__ void __launch_bounds__(256) k_gram(const R* __restrict__ X, const R* __restrict__ Xa,
+__global__ void __launch_bounds__(256) k_gram(const float* __restrict__ X, const float* __restrict__ Xa,
                                               int L, int64_t N, double* __restrict__ part) {
-    __shared__ __align__(16) R zs[GRAM_PIX][GRAM_LDZ];   // pixel-major tile
+    __shared__ __align__(16) float zs[GRAM_PIX][GRAM_LDZ];   // pixel-major tile
     const int tid = threadIdx.x;
     const int bi = tid >> 4, bj = tid & 15;
-    R hi[16], lo[16];
+    float hi[16], lo[16];
 #pragma unroll
     for (int q = 0; q < 16; ++q) {
         hi[q] = 0;
@@ -532,13 +531,13 @@ __global__ void __launch_bounds__(256) k_gram(const R* __restrict__ X, const R* 
     // next tile's values are loaded into registers while the current one is used
     constexpr int PER = MAX_L_NUC * GRAM_PIX / 256;
     const int px0 = tid & (GRAM_PIX - 1), l0 = tid >> 6;
-    R pre[PER];
+    float pre[PER];
     auto fetch = [&](int64_t tile) {
         const int64_t n = tile * GRAM_PIX + px0;
 #pragma unroll
         for (int m = 0; m < PER; ++m) {
             const int l = l0 + 4 * m;
-            R z = 0;
+            float z = 0;
             if (l < L && tile < ntile) {
                 z = X[(int64_t)l * N + n];
                 if (Xa) z += Xa[(int64_t)l * N + n];
@@ -555,12 +554,12 @@ __global__ void __launch_bounds__(256) k_gram(const R* __restrict__ X, const R* 
         fetch(tile + gridDim.x);
 #pragma unroll
         for (int half = 0; half < GRAM_PIX / 32; ++half) {
-            R acc[16];
+            float acc[16];
 #pragma unroll
             for (int q = 0; q < 16; ++q) acc[q] = 0;
 #pragma unroll 4
             for (int px = 32 * half; px < 32 * half + 32; ++px) {
-                R a[4], b[4];
+                float a[4], b[4];
                 ld4(&zs[px][4 * bi], a);
                 ld4(&zs[px][4 * bj], b);
 #pragma unroll
@@ -570,9 +569,9 @@ __global__ void __launch_bounds__(256) k_gram(const R* __restrict__ X, const R* 
             }
 #pragma unroll
             for (int q = 0; q < 16; ++q) {   // (hi, lo) += acc, hi + e = old hi + acc exactly
-                const R sum = hi[q] + acc[q];
-                const R bp = sum - hi[q];
-                const R e = (hi[q] - (sum - bp)) + (acc[q] - bp);
+                const float sum = hi[q] + acc[q];
+                const float bp = sum - hi[q];
+                const float e = (hi[q] - (sum - bp)) + (acc[q] - bp);
                 hi[q] = sum;
                 lo[q] += e;
             }
@@ -867,7 +866,7 @@ hs_status gram_matrix(Plan* p, const void* X, const void* Xadd, cudaStream_t s) 
     if (p->prec == HS_F32 && p->gram_tc && gram_tc_usable(X, Xadd, L, N)) {
         HS_TRY(gram_tc_launch((const float*)X, (const float*)Xadd, L, N, p->part, GRAM_CTAS, p->err_d, &nb, s));
     } else if (p->prec == HS_F32) {
-        k_gram<float><<<GRAM_CTAS, 256, 0, s>>>((const float*)X, (const float*)Xadd, L, N, p->part);
+        k_gram<<<GRAM_CTAS, 256, 0, s>>>((const float*)X, (const float*)Xadd, L, N, p->part);
     } else {
         k_gram_f64<<<GRAM_CTAS, 256, 0, s>>>((const double*)X, (const double*)Xadd, L, N, p->part);
     }
