@@ -172,9 +172,9 @@ __device__ __forceinline__ float two_sum(float& a, float x) {
 //    a third value: ~68 bits of a row's sum s.
 //  * Its root is r + c + c2: r rounded, c the correction by the residual s - r^2, c2 by the
 //    residual of r + c (its own error below 2^-66 of r).
-//  * r times the weight is a pair again. Its high part goes to the FP64 sum (one conversion and one
-//    addition per row, where a root in FP64 took 17 instructions), its low part and the corrections to a
-//    pair that is added at the end.
+//  * r times the weight is a pair again. The high parts of two rows go to the FP64 sum together (one
+//    conversion and one addition, where a root in FP64 took 17 instructions a row), the low parts and
+//    the corrections to a pair that is added at the end.
 // With two values to a row and FP32 pairs for the rows the norm was 2 to 5e-16 off where the plain
 // form and this one are at 1e-16 and below; and the products of a thread's rows (162 at 2048 x 2048), each inside the FP32
 // range, left it together. A lane owns two neighbouring rows at a time and 16 of their channels
@@ -182,8 +182,8 @@ __device__ __forceinline__ float two_sum(float& a, float x) {
 // 512 x 512, L = 32). Rows whose squares or products leave the range in which the pairs are exact
 // (or are not finite) are summed again in FP64. Bound by FP32 issue (24 instructions a coefficient):
 // us per call with the copy to the host, plain form -> two values -> this: 512 x 512, L = 32
-// 410 -> 87 -> 110; 1024 x 1024, L = 1 122 -> 183 for the last two (many rows of one channel).
-__global__ void __launch_bounds__(256) k_l21_norm_exact(const float* __restrict__ A,
+// 410 -> 88 -> 112, L = 10 60 -> 64 (the last two); 1024 x 1024, L = 16 160 -> 212, L = 1 122 -> 110.
+__global__ void __launch_bounds__(256, 4) k_l21_norm_exact(const float* __restrict__ A,
                                                         const float* __restrict__ w_rows, int L, int64_t N,
                                                         double* __restrict__ part) {
     __shared__ double red[32];
@@ -204,6 +204,7 @@ __global__ void __launch_bounds__(256) k_l21_norm_exact(const float* __restrict_
                                   : make_float2(0.f, 0.f);
 #pragma unroll
             for (int c = 0; c < 16; ++c) {
+                if (l0 + c >= L) break;
                 const float q[2] = {v[c].x, v[c].y};
 #pragma unroll
                 for (int k = 0; k < 2; ++k) {
@@ -215,6 +216,7 @@ __global__ void __launch_bounds__(256) k_l21_norm_exact(const float* __restrict_
                 }
             }
         }
+        float both = 0.f;   // high parts of the two rows
 #pragma unroll
         for (int k = 0; k < 2; ++k) {
             const float s = hi[k];
@@ -235,7 +237,7 @@ __global__ void __launch_bounds__(256) k_l21_norm_exact(const float* __restrict_
                 const float e = two_sum(slo, __fmaf_rn(r, wr, -p));
                 const float f = two_sum(slo, cw);
                 sll = __fadd_rn(sll, __fadd_rn(__fadd_rn(e, f), fmaf(c2, wr, __fmaf_rn(c, wr, -cw))));
-                acc += (double)p;
+                sll = __fadd_rn(sll, two_sum(slo, two_sum(both, p)));
             } else {
                 double d = 0.0;
                 if (mx[k] != 0.f || !(s == 0.f))   // not a zero row
@@ -246,6 +248,7 @@ __global__ void __launch_bounds__(256) k_l21_norm_exact(const float* __restrict_
                 acc += sqrt(d) * (double)wr;
             }
         }
+        acc += (double)both;
     }
     acc = block_sum(acc + ((double)slo + (double)sll), red);
     if (threadIdx.x == 0) part[blockIdx.x] = acc;
@@ -349,7 +352,7 @@ hs_status l21_norm(Plan* p, const void* A, const void* w_rows, double* out_dev, 
     const int64_t N = p->N();
     int nb = 512;
     if (p->prec == HS_F32 && N % 2 == 0 && (uintptr_t)A % 8 == 0) {
-        nb = (int)std::min<int64_t>(nblk(NB * (N / 2), 256), 152 * 5);   // 48 registers: 5 CTAs to an SM
+        nb = (int)std::min<int64_t>(nblk(NB * (N / 2), 256), 152 * 4);   // 64 registers: 4 CTAs to an SM
         k_l21_norm_exact<<<nb, 256, 0, s>>>((const float*)A, (const float*)w_rows, p->g.L, N, p->part);
     } else if (p->prec == HS_F32)
         k_l21_norm<float><<<nb, 256, 0, s>>>((const float*)A, (const float*)w_rows, p->g.L, N, p->part);
