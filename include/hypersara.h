@@ -71,7 +71,9 @@ typedef enum { HS_F32 = 0, HS_F64 = 1 } hs_prec;
  * Kahan-compensated sums (FP32 plans). Without it grids of at least 64 x 64
  * cells use the register sweep (uncompensated, faster) and smaller grids add 4
  * non-overlapping windows per warp pass into per-warp tiles. Every form sums in
- * a fixed order, so all are bitwise reproducible. */
+ * a fixed order, so a plan's results are bitwise reproducible; plans tuned in
+ * different processes may take work lists that add in another order
+ * (HS_PLAN_NO_TUNE fixes them). */
 #define HS_PLAN_COMPENSATED 1u
 /* FP32 plans: form the nuclear prox's L x L Gram matrix with register-blocked
  * FMA on the CUDA cores instead of the tensor cores (tcgen05 BF16 products of
@@ -104,7 +106,8 @@ HS_API const char* hs_last_error(void);
 
 /*
  * hs_plan_create - measurement setup for one wideband problem (Sec. 2.1).
- *   nx, ny        image size; powers of two in [16, 2048], divisible by 2^wavelet_levels.
+ *   nx, ny        image size in [16, 2048]: powers of two, or 3 or 5 times a power of two and
+ *                 multiples of 16; divisible by 2^wavelet_levels.
  *   L             number of channels, 1..1024 (the nuclear-norm prox needs L <= 64).
  *   vis_offsets   HOST array of L+1 int64: visibilities of channel l are
  *                 [vis_offsets[l], vis_offsets[l+1]); vis_offsets[0] = 0,
