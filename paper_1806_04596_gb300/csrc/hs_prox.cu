@@ -225,7 +225,8 @@ __global__ void __launch_bounds__(256, 4) k_l21_norm_exact(const float* __restri
             float r = s * y;
             r = fmaf(h, fmaf(-r, r, s), r);
             const float p = __fmul_rn(r, wr);
-            if (s >= 0x1p-85f && s <= 0x1p126f && fabsf(p) >= 0x1p-60f && fabsf(p) <= 0x1p120f) {
+            // (a weight of zero leaves only zeros: rows that are masked out stay on this side)
+            if (s >= 0x1p-85f && s <= 0x1p126f && (fabsf(p) >= 0x1p-60f || wr == 0.f) && fabsf(p) <= 0x1p120f) {
                 const float q = __fmul_rn(r, r);
                 float m = __fsub_rn(s, q);   // s - r^2 = m + rest (the difference is exact)
                 float rest = two_sum(m, -__fmaf_rn(r, r, -q));
