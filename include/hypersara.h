@@ -383,8 +383,9 @@ typedef struct {
  * at zero. The state keeps references to params->w_nuc / w_l21, which must stay
  * valid while it is used. FP32 states with the nuclear prior iterate on a second layout of the
  * plan's coverage (about 20 bytes per visibility, shared by the plan's states; kept by the plan
- * unless a device limit is set); where that does not fit they iterate on the plan's
- * own, with sums in another order. Errors: HS_ERR_ARG, HS_ERR_NOMEM, HS_ERR_CUDA.
+ * unless a device limit is set); where that does not fit, or under a device limit takes more than
+ * 48 bytes per pixel and channel, they iterate on the plan's own, with sums in another
+ * order. Errors: HS_ERR_ARG, HS_ERR_NOMEM, HS_ERR_CUDA.
  */
 HS_API hs_status hs_pd_state_create(hs_plan_t plan, const void* Y, const double* eps,
                              const hs_pd_params* params, hs_pd_state_t* out, void* stream);

@@ -1065,12 +1065,24 @@ int64_t plane_bytes(Plan* p) {
     return c ? c->device_bytes : 0;
 }
 
+// Under a device limit the layout only takes what the wavelet scratch between levels leaves
+// of the two coefficient cubes it could be (48 bytes per pixel and channel, about 1.7 to 2
+// visibilities), so that as many states and plans fit as beside one layout. Without the rule the
+// first state of a denser plan took the room of the second.
+static hs_status plane_room(const Plan* p, int64_t bytes) {
+    const int64_t room = 2 * NW * p->g.L * (p->N() - p->N() / 4) * (int64_t)p->rsize();
+    if (device_limit() == 0 || bytes <= room) return HS_OK;
+    return fail(HS_ERR_NOMEM, "whole-plane layout: %lld bytes, %lld left for it under the device limit", (long long)bytes,
+                (long long)room);
+}
+
 static hs_status make_plane(Plan* p, std::shared_ptr<Plan>* out, cudaStream_t s) {
     std::lock_guard<std::mutex> lock(p->plane_mu);
     *out = p->plane.lock();
     if (*out) return HS_OK;
     if (p->prec != HS_F32 || (int64_t)p->uv_h.size() != 2 * p->M_total)
         return fail(HS_ERR_STATE, "whole-plane layout: the plan keeps no coverage");
+    HS_TRY(plane_room(p, 16 * p->M_total));   // coordinates, permutation and list entries: at least
     std::shared_ptr<Plan> c(new Plan(), [](Plan* q) {
         plan_free(q);
         delete q;
@@ -1137,6 +1149,7 @@ static hs_status make_plane(Plan* p, std::shared_ptr<Plan>* out, cudaStream_t s)
         HS_TRY(e);
         HS_CHECK_CUDA(ce);
     }
+    HS_TRY(plane_room(p, c->device_bytes));
     c->grid = p->grid;
     c->tmp = p->tmp;
     c->vis = p->vis;
