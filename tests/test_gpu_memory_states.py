@@ -1,6 +1,7 @@
 """Several solver states under hs_set_device_limit: as many FP32 states with the nuclear prior, and
 their staging for host data, fit beside a plan as would beside one set of lists and wavelet
-scratch of two coefficient cubes, at sparse and at dense coverage."""
+scratch of two coefficient cubes, at sparse and at dense coverage (in between the first state's second layout
+would fit in the room of the second state)."""
 
 import numpy as np
 import pytest
@@ -10,7 +11,7 @@ from gpu_util import dev, host, make_plan, ragged_case, rel
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("M", [(2000, 1503, 0, 911), (60000, 40000, 50000, 0)])
+@pytest.mark.parametrize("M", [(2000, 1503, 0, 911), (20000, 15000, 20000, 0), (60000, 40000, 50000, 0)])
 def test_two_states_and_host_data_fit_under_a_limit(cuda_device, M):
     import torch
     import __graft_entry__ as ge
