@@ -382,7 +382,7 @@ typedef struct {
  * L unless the plan has blocks; copied). All primal and dual variables start
  * at zero. The state keeps references to params->w_nuc / w_l21, which must stay
  * valid while it is used. FP32 states with the nuclear prior iterate on a second layout of the
- * plan's coverage (about 20 bytes per visibility, shared by the plan's states; kept by the plan
+ * plan's coverage (20 to 55 bytes per visibility, shared by the plan's states; kept by the plan
  * unless a device limit is set); where that does not fit, or under a device limit takes more than
  * 48 bytes per pixel and channel, they iterate on the plan's own, with sums in another
  * order. Errors: HS_ERR_ARG, HS_ERR_NOMEM, HS_ERR_CUDA.
